@@ -76,6 +76,51 @@ extern "C" void gf_query_opts_default(gf_query_opts *o) {
     o->precision = GF_FP32;
 }
 
+// ---------------------------------------------------------------- per-call scratch
+
+namespace {
+
+constexpr int MAX_DEVICES = 64;
+constexpr uint64_t SCRATCH_KEEP = 1ull << 30;  // bytes a pool keeps across synchronizations
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[MAX_DEVICES] = {};
+int g_live_forests = 0;  // under g_pool_mu
+
+cudaError_t scratch_pool(cudaMemPool_t *pool) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> g(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+        uint64_t keep = SCRATCH_KEEP;
+        if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+            cudaMemPoolDestroy(p);
+            return e;
+        }
+        g_pool[dev] = p;
+    }
+    *pool = g_pool[dev];
+    return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t gf_scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
+    cudaMemPool_t pool = nullptr;
+    const cudaError_t e = scratch_pool(&pool);
+    return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, st) : e;
+}
+
+void gf_scratch_free(void *p, cudaStream_t st) { cudaFreeAsync(p, st); }
+
 // ---------------------------------------------------------------- forest storage
 
 // Destroy everything the forest owns (tolerates partially built forests).
@@ -90,6 +135,12 @@ static void forest_release(gf_forest *F) {
     cudaFree(F->scale8);
     cudaFree(F->x8n);
     cudaFree(F->U);
+    if (F->live) {
+        std::lock_guard<std::mutex> g(g_pool_mu);
+        if (--g_live_forests == 0)
+            for (cudaMemPool_t p : g_pool)
+                if (p) cudaMemPoolTrimTo(p, 0);
+    }
     delete F;
 }
 
@@ -146,6 +197,11 @@ int gf_forest_alloc(gf_forest **out, const float *X, int64_t n, int32_t d, int32
     if ((r = gf_dmalloc((void **)&F->nodes, (size_t)T * nn * sizeof(int2)))) { forest_release(F); return r; }
     if ((r = gf_dmalloc((void **)&F->perm, (size_t)T * n * 4))) { forest_release(F); return r; }
     F->device_bytes = (borrow ? 0 : (int64_t)n * F->ldx * 4) + (int64_t)(T * nn * sizeof(int2)) + (int64_t)T * n * 4;
+    {
+        std::lock_guard<std::mutex> g(g_pool_mu);
+        F->live = true;
+        ++g_live_forests;
+    }
     *out = F;
     return GF_OK;
 }
@@ -431,6 +487,7 @@ extern "C" int gf_query_ex(const gf_forest *F, const float *Q, int64_t m, int32_
     if (o->checks < 0 || !(o->eps >= 0.0)) return gf_fail(GF_EINVAL, "checks < 0 or eps < 0");
     x.leaf_budget = leaf_budget_of(F, o->checks, o->eps);
     x.events = (cudaEvent_t *)o->events;
+    x.shaped = o->warps_per_cta > 0 || o->ctas_per_sm > 0 || o->rows_in_flight > 0 || warps > 8;
     if (x.leaf_budget > 0) {
         if (((unsigned long long)F->T << F->L) > 0xffffffffull)
             return gf_fail(GF_EUNSUPPORTED, "priority search needs T * 2^L <= 2^32");

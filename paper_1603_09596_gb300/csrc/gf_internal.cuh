@@ -44,6 +44,7 @@ struct gf_forest {
     int32_t tune_R[3] = {0, 64, 128};
     int32_t tune_G[3] = {0, 0, 0};  // rows in flight per warp, 0 = kernel default
     int64_t device_bytes = 0;
+    bool live = false;  // counted among the forests that keep the scratch pool's memory
 };
 
 // Limits of the tuning values (gf_forest_set_tuning, forest files): an SM runs at most 32 CTAs,
@@ -141,6 +142,7 @@ struct QueryExtra {
     int32_t order = GF_ORDER_AUTO;
     int32_t leaf_budget = 0;  // leaves per query for the priority search (0: one per tree)
     cudaEvent_t *events = nullptr;  // recorded around the scoring kernel's launches (timing)
+    bool shaped = false;            // the caller (or the forest's tuning) asks for a CTA shape of the one-CTA kernels
 };
 
 // Record events[i] on st when the caller asked for timing events.
@@ -180,6 +182,20 @@ bool gf_leaf_preferred(const gf_forest *F, int64_t m, int32_t k, int32_t precisi
 // Why the leaf-major path cannot run this query (nullptr: it can).
 const char *gf_leaf_unsupported(const gf_forest *F, int64_t m, int32_t k, int32_t precision, int32_t R,
                                 const QueryExtra &x);
+
+// Staged per-query path (gf_list.cu).  usable: its selection and shared memory hold this query.
+// launch: *ran = false (and GF_OK) when its scratch could not be allocated.
+bool gf_list_usable(const gf_forest *F, int64_t m, int32_t k, int32_t precision, int32_t R, const QueryExtra &x);
+int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision, int32_t R,
+                   cudaStream_t st, int64_t *ids, float *dists, const QueryExtra &x, bool *ran);
+// order[0..m) = the queries of okeys (leaf << 32 | query) sorted, in chunks of 16,384
+cudaError_t gf_sort_order(int64_t m, const unsigned long long *okeys, int *order, cudaStream_t st);
+
+// Per-call device scratch, stream-ordered, from a pool of the library's own that keeps up to 1 GiB
+// between calls (the default pool gives everything back at each synchronization, and mapping it
+// again costs 0.2 ms a call); given back when the last forest is freed.
+cudaError_t gf_scratch_alloc(void **p, size_t bytes, cudaStream_t st);
+void gf_scratch_free(void *p, cudaStream_t st);
 
 int gf_launch_query(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision,
                     int32_t R, int32_t warps, int32_t ctas_per_sm, cudaStream_t s, int64_t *ids,

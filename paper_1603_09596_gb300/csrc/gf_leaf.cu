@@ -1267,7 +1267,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
         if ((size_t)workspace_bytes < W.total)
             return gf_fail(GF_EINVAL, "workspace of %lld bytes, %zu needed", (long long)workspace_bytes, W.total);
     } else {
-        cudaError_t e = cudaMallocAsync((void **)&ws, W.total, st);
+        cudaError_t e = gf_scratch_alloc((void **)&ws, W.total, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return gf_fail(GF_ENOMEM, "leaf-major workspace of %zu bytes: %s", W.total, cudaGetErrorString(e));
@@ -1275,7 +1275,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
         own = true;
     }
     auto fail = [&](cudaError_t e, const char *what) {
-        if (own) cudaFreeAsync(ws, st);
+        if (own) gf_scratch_free(ws, st);
         return gf_cuda_fail(e, what);
     };
     int *bcnt = (int *)(ws + W.bcnt), *bfill = (int *)(ws + W.bfill);
@@ -1298,7 +1298,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     // the leaves of every query: the descents, or the priority search's lists
     int r = prio ? gf_launch_prio_leaves(F, Q, m, S, (unsigned *)leaf, pn, st) : gf_descend(F, Q, m, leaf, st);
     if (r) {
-        if (own) cudaFreeAsync(ws, st);
+        if (own) gf_scratch_free(ws, st);
         return r;
     }
     PairSource P;
@@ -1382,7 +1382,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "k_leaf_merge launch");
     // a caller's workspace is handed back all zero, as the streaming kernel expects it
     if (!own && (e = cudaMemsetAsync(ws, 0, W.total, st)) != cudaSuccess) return fail(e, "workspace clear");
-    if (own) cudaFreeAsync(ws, st);
+    if (own) gf_scratch_free(ws, st);
     return GF_OK;
 }
 
