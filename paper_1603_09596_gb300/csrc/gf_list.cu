@@ -4,22 +4,24 @@
 //   1. the leaves of every (query, tree): gf_descend, or one warp per pair (k_list_descend), or the
 //      priority search's list;
 //   2. admit: the points of a query's leaves are written to its candidate list once each (the "seen"
-//      array of Sec. 2.3): through a hash set in shared memory, one CTA a query, or through a bitmap
-//      over the point ids in device memory, a warp per 128 positions of a leaf;
+//      array of Sec. 2.3): through a hash set or a bitmap over the point ids in shared memory, one CTA
+//      a query; for a few queries of many candidates, or too many points for that, through a bitmap in
+//      device memory, a warp per 128 positions of a leaf;
 //   3. score (k_list_score): CTAs take blocks of rows of the lists, a warp G rows at a time;
 //   4. select (k_list_select): one CTA a query finds the `keep` smallest keys (distance, id), rescores
 //      a screen's shortlist in float32 and writes the k nearest.
+// Calls too small for five launches run the same steps in one (k_list_one).
 // A row's distance is warp_dist_g's, the same arithmetic in the same order as in the other per-query
 // kernels, and a key holds (distance, id), so the answers are theirs bit for bit.
 //
 // Why: a query that is one CTA's alone reads its rows at that CTA's rate, and its descent,
 // de-duplication and sorts stand between the reads.  Here step 3 is a flat pass over all rows of the
 // batch that the whole chip shares.  Microseconds a call on one GB300, the one-CTA kernels -> this:
-//   1 query, 10^6 x 960, T = 32, p = 1024, bf16 (10.9k rows)        1004 -> 41   (streaming)
-//   199 queries, 5 10^5 x 960, T = 32, p = 512, bf16 (5.6k rows)     774 -> 357  (streaming)
-//   27 queries, 5 10^4 x 512, T = 16, p = 256, float32               164 -> 40   (sort)
-//   10^4 queries, 10^6 x 960, T = 32, p = 64, bf16 (1.24k rows)     8822 -> 3216 (sort)
-//   5003 queries, 7 10^5 x 101, T = 32, p = 64, float32              902 -> 462  (sort)
+//   1 query, 10^6 x 960, T = 32, p = 1024, bf16 (10.9k rows)         856 -> 33   (streaming)
+//   199 queries, 5 10^5 x 960, T = 32, p = 512, bf16 (5.6k rows)     779 -> 328  (streaming)
+//   27 queries, 5 10^4 x 512, T = 16, p = 256, float32               165 -> 39   (sort)
+//   10^4 queries, 10^6 x 960, T = 32, p = 64, bf16 (1.24k rows)     8798 -> 3037 (sort)
+//   5003 queries, 7 10^5 x 101, T = 32, p = 64, float32              890 -> 419  (sort)
 // The scoring step is bound by the row loads: 9.8 TB/s of rows at 10^4 queries (most from L2, whose
 // register loads peak at 10.6 TB/s), 7.2 TB/s at 199 queries (HBM).
 #include "gf_internal.cuh"
@@ -35,7 +37,11 @@ constexpr int KEEP_MAX = 128;      // longest k or R the selection keeps (it sor
 constexpr int GROUPS = 256;        // groups of keys whose minima bound the keep-th key
 constexpr int SEL_BUF = 1024;      // keys at or below that bound the selection holds
 constexpr int HASH_MAX = 16384;    // slots of the shared-memory hash set (at least twice the ids)
+constexpr int MAP_MAX = 1800000;   // points whose bitmap fits shared memory (225,000 bytes)
+constexpr int FEW = 16;            // batches up to here spread a query's admission over many CTAs
 constexpr int SEG = 128;           // positions of a leaf a warp admits at once (four a lane)
+constexpr int ONE_MAX = 640000;    // candidates of a call that runs in one launch,
+constexpr int ONE_BYTES = 768 << 10;  // and bytes of a query's rows there, with fewer queries than SMs
 constexpr int ORDER_MIN = 512;     // batches from here on are walked in the order of tree 0's leaves
 
 // The leaves of the batch: leaf[q][T] (one per tree) or the priority search's lists.
@@ -63,18 +69,13 @@ __device__ __forceinline__ int leaf_of(const ForestView &F, const Leaves &V, lon
     return (int)(hi - lo);
 }
 
-// One warp per (query, tree): the warp loads the five-level subtree below the current node at once
-// (lane i: node i in breadth-first order, with the query's coordinate) and walks it through shuffles,
-// so a path of L nodes costs ceil(L / 5) rounds of dependent loads instead of L.  For batches of a
-// few thousand pairs, where the chip has warps to spare and the latency of the chain is what counts.
-__global__ void __launch_bounds__(128) k_list_descend(ForestView F, const float *__restrict__ Q, long long pairs,
-                                                      int *leaf) {
+// The leaf of tree t that query q reaches (Eq. 1), by a whole warp: it loads the five-level subtree
+// below the current node at once (lane i: node i in breadth-first order, with the query's coordinate)
+// and walks it in the ballot of the comparisons, so a path of L nodes costs ceil(L / 5) rounds of
+// dependent loads instead of L.  For batches of a few thousand (query, tree) pairs, where the chip has
+// warps to spare and the latency of the chain is what counts.
+__device__ __forceinline__ int warp_descend(const ForestView &F, int t, const float *__restrict__ q) {
     const int lane = threadIdx.x & 31;
-    const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (g >= pairs) return;
-    const long long qi = g / F.T;
-    const int t = (int)(g - qi * F.T);
-    const float *q = Q + qi * F.d;
     const int2 *nodes = F.nodes + (size_t)t * F.nnodes;
     const int lv = 31 - __clz(lane + 1);  // lane's level in the subtree (lanes 0..30)
     int j = 0;
@@ -88,64 +89,95 @@ __global__ void __launch_bounds__(128) k_list_descend(ForestView F, const float 
         const unsigned lefts = __ballot_sync(FULL, left);
         int bi = 0;
         for (int l = 0; l < 5 && j < F.nnodes; ++l) {
-            const int right = (lefts >> bi) & 1u ? 1 : 2;
-            j = 2 * j + right;
-            bi = 2 * bi + right;
+            const int side = (lefts >> bi) & 1u ? 1 : 2;
+            j = 2 * j + side;
+            bi = 2 * bi + side;
         }
     }
-    if (lane == 0) leaf[g] = j - F.nnodes;
+    return j - F.nnodes;
+}
+
+__global__ void __launch_bounds__(128) k_list_descend(ForestView F, const float *__restrict__ Q, long long pairs,
+                                                      int *leaf) {
+    const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (g >= pairs) return;
+    const long long qi = g / F.T;
+    const int b = warp_descend(F, (int)(g - qi * F.T), Q + qi * F.d);
+    if ((threadIdx.x & 31) == 0) leaf[g] = b;
 }
 
 // ---------------------------------------------------------------- admission
 
-// One CTA per query: every id of its leaves goes into a hash set in shared memory (open addressing,
-// linear probing; the table has at least twice as many slots as ids, so a probe ends) and, when it
-// was not there, to the query's list.
-__global__ void __launch_bounds__(256) k_list_admit_hash(ForestView F, Leaves V, long long q0, const int *__restrict__ order,
-                                                         int slots, int cap, unsigned long long *keys, int *cnt) {
+// Whether `id` is new to the shared-memory set, adding it.
+template <bool BITS>
+__device__ __forceinline__ bool seen_first(int *table, int words, int id) {
+    if (BITS) {
+        const int bit = 1 << (id & 31);
+        return !(atomicOr(table + (id >> 5), bit) & bit);
+    }
+    unsigned h = ((unsigned)id * 2654435769u) >> (__clz(words) + 1);  // the hash's top log2(words) bits
+    for (;;) {
+        const int old = atomicCAS(table + h, -1, id);
+        if (old == -1) return true;
+        if (old == id) return false;
+        h = (h + 1) & (unsigned)(words - 1);
+    }
+}
+
+// One CTA per query: every id of its leaves is tested and set in shared memory and, when it was not
+// there, written to the query's list.  BITS: a bitmap over the point ids; else a hash set (open
+// addressing, linear probing; the table has at least twice as many slots as ids, so a probe ends).
+// A warp has eight ids a lane in flight: of one leaf, or (SHORT: leaves of at most 64) of four.
+template <bool BITS, bool SHORT, int NT>
+__global__ void __launch_bounds__(NT) k_list_admit(ForestView F, Leaves V, long long q0, const int *__restrict__ order,
+                                                   int words, int cap, unsigned long long *keys, int *cnt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    int *table = reinterpret_cast<int *>(smem_raw);
+    int *table = reinterpret_cast<int *>(smem_raw);  // [words], a multiple of four
     __shared__ int count;
     const long long w0 = blockIdx.x;
     const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
-    for (int i = threadIdx.x; i < slots / 4; i += blockDim.x) reinterpret_cast<int4 *>(table)[i] = make_int4(-1, -1, -1, -1);
+    const int none = BITS ? 0 : -1;
+    for (int i = threadIdx.x; i < words / 4; i += NT) reinterpret_cast<int4 *>(table)[i] = make_int4(none, none, none, none);
     if (threadIdx.x == 0) count = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int shift = __clz(slots) + 1;  // a multiplicative hash's top log2(slots) bits
     unsigned long long *out = keys + w0 * cap;
-    auto admit = [&](int id) {
-        bool fresh = false;
-        if (id >= 0) {
-            unsigned h = ((unsigned)id * 2654435769u) >> shift;
-            for (;;) {
-                const int old = atomicCAS(table + h, -1, id);
-                if (old == -1) { fresh = true; break; }
-                if (old == id) break;
-                h = (h + 1) & (unsigned)(slots - 1);
-            }
-        }
-        __syncwarp();
-        const unsigned bl = __ballot_sync(FULL, fresh);
-        int at = 0;
-        if (lane == 0 && bl) at = atomicAdd(&count, __popc(bl));
-        at = __shfl_sync(FULL, at, 0);
-        if (fresh) out[at + __popc(bl & lt)] = (unsigned)id;
-    };
-    // two leaves of a warp in flight
-    for (int s = w; s < V.S; s += 2 * nw) {
-        long long b0, b1 = 0;
-        const int c0 = leaf_of(F, V, qi, s, b0);
-        const int c1 = s + nw < V.S ? leaf_of(F, V, qi, s + nw, b1) : 0;
-        for (int i = lane; i - lane < max(c0, c1); i += 64) {
-            int id[4];
-            id[0] = i < c0 ? __ldg(F.perm + b0 + i) : -1;
-            id[1] = i < c1 ? __ldg(F.perm + b1 + i) : -1;
-            id[2] = i + 32 < c0 ? __ldg(F.perm + b0 + i + 32) : -1;
-            id[3] = i + 32 < c1 ? __ldg(F.perm + b1 + i + 32) : -1;
+    constexpr int PER = SHORT ? 4 : 1;  // leaves at once
+    constexpr int E = 8 / PER;          // ids a lane of each
+    for (int s = w * PER; s < V.S; s += NT / 32 * PER) {
+        long long base[PER];
+        int c[PER], longest = 0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) admit(id[u]);
+        for (int h = 0; h < PER; ++h) {
+            base[h] = 0;
+            c[h] = s + h < V.S ? leaf_of(F, V, qi, s + h, base[h]) : 0;
+            longest = max(longest, c[h]);
+        }
+        for (int i0 = 0; i0 < longest; i0 += 32 * E) {
+            int id[8];
+            unsigned bl[8];
+            int total = 0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int i = i0 + lane + 32 * (u % E);
+                id[u] = i < c[u / E] ? __ldg(F.perm + base[u / E] + i) : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool fresh = id[u] >= 0 && seen_first<BITS>(table, words, id[u]);
+                __syncwarp();
+                bl[u] = __ballot_sync(FULL, fresh);
+                total += __popc(bl[u]);
+            }
+            int at = 0;
+            if (lane == 0 && total) at = atomicAdd(&count, total);
+            at = __shfl_sync(FULL, at, 0);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if ((bl[u] >> lane) & 1u) out[at + __popc(bl[u] & lt)] = (unsigned)id[u];
+                at += __popc(bl[u]);
+            }
         }
     }
     __syncthreads();
@@ -231,11 +263,120 @@ __global__ void __launch_bounds__(256, 2) k_list_score(ForestView F, const float
 
 // ---------------------------------------------------------------- selection and rerank
 
-// The `keep` smallest of a query's C keys.  The keys are dealt to GROUPS groups; the keep-th
-// smallest group minimum bounds the keep-th key from above (each of the keep groups holds a key at
-// or below it), and few other keys lie below it (about keep of them in all when the keys' order is
-// unrelated to their size): those are gathered and sorted.  A list in an order that leaves more than
-// SEL_BUF below the bound goes through the radix select.
+// Ascending sort of the distinct keys a[0..n) by counting, for every key, the smaller ones (three
+// barriers; a bitonic sort of 64 keys takes 21): up to one key a thread.  More go to the bitonic sort.
+__device__ void sort_distinct(unsigned long long *a, int n) {
+    if (n > (int)blockDim.x) {
+        sort_keys(a, n);
+        return;
+    }
+    __syncthreads();
+    const unsigned long long key = (int)threadIdx.x < n ? a[threadIdx.x] : 0ull;
+    int rank = 0;
+    if ((int)threadIdx.x < n) {
+        for (int j = 0; j < n; ++j) rank += a[j] < key;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < n) a[rank] = key;
+    __syncthreads();
+}
+
+struct SelectShared {
+    unsigned hist[256];
+    unsigned long long pref, bound;
+    int sid[KEEP_MAX];
+    int nheld, hs;
+};
+
+// The `keep` smallest (or all, if fewer) of the C distinct keys kq[0..C), ascending in a[] (shared
+// memory, SEL_BUF entries, not overlapping kq); returns their number.  The keys are dealt to GROUPS
+// groups; the keep-th smallest group minimum bounds the keep-th key from above (each of the keep
+// groups holds a key at or below it), and few other keys lie below it (about keep in all when the
+// keys' order is unrelated to their size): those are gathered and sorted.  A list in an order that
+// leaves more than SEL_BUF below the bound goes through the radix select.  Up to NT KPT keys are read
+// once, into registers.
+template <int NT, int KPT>
+__device__ int select_keys(const unsigned long long *kq, int C, int keep, unsigned long long *a, SelectShared &S) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const bool held = C <= NT * KPT;
+    unsigned long long v[KPT];
+    if (held) {
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) v[u] = tid + u * NT < C ? kq[tid + u * NT] : KEY_NONE;
+    }
+    unsigned long long bound = KEY_NONE;
+    if (tid == 0) S.nheld = 0;
+    if (C > GROUPS) {
+        unsigned long long mn = KEY_NONE;
+        if (held) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) mn = v[u] < mn ? v[u] : mn;
+        } else {
+#pragma unroll 8
+            for (int i = tid; i < C; i += NT) {
+                const unsigned long long x = kq[i];
+                mn = x < mn ? x : mn;
+            }
+        }
+        if (NT > GROUPS) {
+            if (tid >= GROUPS) a[tid] = mn;
+            __syncthreads();
+            if (tid < GROUPS) {
+#pragma unroll
+                for (int o = GROUPS; o < NT; o += GROUPS) mn = a[tid + o] < mn ? a[tid + o] : mn;
+            }
+        }
+        if (tid < GROUPS) a[tid] = mn;
+        __syncthreads();
+        if (tid < GROUPS) {
+            int rank = 0;
+#pragma unroll 8
+            for (int j = 0; j < GROUPS; ++j) rank += a[j] < mn;
+            if (rank == keep - 1) S.bound = mn;
+        }
+    }
+    __syncthreads();
+    if (C > GROUPS) bound = S.bound;
+    auto put = [&](unsigned long long x) {
+        const bool in = x != KEY_NONE && x <= bound;
+        const unsigned bl = __ballot_sync(FULL, in);
+        if (bl) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&S.nheld, __popc(bl));
+            at = __shfl_sync(FULL, at, 0) + __popc(bl & lt);
+            if (in && at < SEL_BUF) a[at] = x;
+        }
+    };
+    auto gather = [&]() {
+        if (held) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) put(v[u]);
+        } else {
+            for (int b0 = 0; b0 < C; b0 += 4 * NT) {
+                unsigned long long x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = b0 + u * NT + tid < C ? kq[b0 + u * NT + tid] : KEY_NONE;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) put(x[u]);
+            }
+        }
+    };
+    gather();
+    __syncthreads();
+    if (S.nheld > SEL_BUF) {  // (uniform)
+        bound = gfdev::block_select(kq, C, keep - 1, S.hist, &S.pref, &S.hs);
+        if (tid == 0) S.nheld = 0;
+        __syncthreads();
+        gather();
+        __syncthreads();
+    }
+    const int n = S.nheld;
+    sort_distinct(a, n);
+    return min(keep, n);
+}
+
+// One CTA per query: the keep best of its list, a screen's shortlist rescored in float32, the k nearest.
 template <int NCF, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_list_select(ForestView F, const float *__restrict__ Q, long long q0, int k, int keep,
                                                       int rerank, const int *__restrict__ order, int cap,
@@ -244,87 +385,139 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_list_select(ForestVie
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long *a = reinterpret_cast<unsigned long long *>(smem_raw);  // [SEL_BUF]
     float *qs = reinterpret_cast<float *>(a + SEL_BUF);                        // [ldq], rerank only
-    __shared__ int sid[KEEP_MAX];
-    __shared__ unsigned hist[256];
-    __shared__ unsigned long long pref;
-    __shared__ int nheld, hs;
+    __shared__ SelectShared S;
     const long long w0 = blockIdx.x;
     const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
     const int C = cnt[w0];
-    const unsigned long long *kq = keys + w0 * cap;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    const unsigned lt = (1u << lane) - 1u;
     if (rerank) load_query(Q + qi * F.d, F.d, qs);
-    unsigned long long bound = KEY_NONE;
-    if (C > GROUPS) {
-        unsigned long long mn = KEY_NONE;
-#pragma unroll 4
-        for (int i = tid; i < C; i += nt) {
-            const unsigned long long v = kq[i];
-            mn = v < mn ? v : mn;
-        }
-        a[tid] = mn;
-        __syncthreads();
-        if (tid < GROUPS) {
-            for (int o = tid + GROUPS; o < nt; o += GROUPS) mn = a[o] < mn ? a[o] : mn;
-        }
-        __syncthreads();
-        if (tid < GROUPS) a[tid] = mn;
-        block_sort<unsigned long long>(a, GROUPS);
-        bound = a[keep - 1];
-        __syncthreads();
-    }
-    if (tid == 0) nheld = 0;
-    __syncthreads();
-    auto gather = [&]() {
-        for (int b0 = 0; b0 < C; b0 += 4 * nt) {
-            unsigned long long v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = b0 + u * nt + tid;
-                v[u] = i < C ? kq[i] : KEY_NONE;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool in = v[u] != KEY_NONE && v[u] <= bound;
-                const unsigned bl = __ballot_sync(FULL, in);
-                if (bl) {
-                    int at = 0;
-                    if (lane == 0) at = atomicAdd(&nheld, __popc(bl));
-                    at = __shfl_sync(FULL, at, 0) + __popc(bl & lt);
-                    if (in && at < SEL_BUF) a[at] = v[u];
-                }
-            }
-        }
-    };
-    gather();
-    __syncthreads();
-    if (nheld > SEL_BUF) {  // (uniform: nheld is shared)
-        bound = gfdev::block_select(kq, C, keep - 1, hist, &pref, &hs);
-        if (tid == 0) nheld = 0;
-        __syncthreads();
-        gather();
-        __syncthreads();
-    }
-    const int n = nheld;
-    sort_keys(a, n);
-    const int kn = min(keep, n);
+    const int kn = select_keys<NT, NT == 256 ? 8 : 24>(keys + w0 * cap, C, keep, a, S);
     if (rerank) {
-        for (int j = tid; j < kn; j += nt) sid[j] = (int)(unsigned)(a[j] & 0xffffffffu);
+        for (int j = threadIdx.x; j < kn; j += NT) S.sid[j] = (int)(unsigned)(a[j] & 0xffffffffu);
         __syncthreads();
-        rescore_f32<NCF>(F, qs, sid, kn, a);
-        sort_keys(a, kn);
+        rescore_f32<NCF>(F, qs, S.sid, kn, a);
+        sort_distinct(a, kn);
     }
     write_topk(a, kn, k, ids + qi * k, dists + qi * k);
-    if (tid == 0 && ncand_out) ncand_out[qi] = C;
+    if (threadIdx.x == 0 && ncand_out) ncand_out[qi] = C;
 }
 
-// order keys (tree-0 leaf, query) of the batch
-__global__ void k_list_order_keys(Leaves V, int L, long long m, unsigned long long *okeys) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    const unsigned b = V.plist ? V.plist[i * V.S] & ((1u << L) - 1u) : (unsigned)V.leaf[i * V.S];
-    okeys[i] = ((unsigned long long)b << 32) | (unsigned long long)(i & 0xffffffffll);
+// The whole search of a query of at most SEL_BUF candidates in one launch, one CTA a query, for calls
+// too small for the launches of the staged steps to pay.  Every warp descends its trees and admits
+// their leaves' ids at once; the rows are scored G at a time a warp and selected as above.
+template <int PREC, int NC, int NCF, int G>
+__global__ void __launch_bounds__(256) k_list_one(ForestView F, const float *__restrict__ Q, int k, int keep, int words,
+                                                  long long *ids, float *dists, int *ncand_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned long long *a = reinterpret_cast<unsigned long long *>(smem_raw);  // [SEL_BUF]
+    unsigned long long *kq = a + SEL_BUF;                                      // [SEL_BUF]
+    float *qs = reinterpret_cast<float *>(kq + SEL_BUF);                       // [ldq]
+    int *table = reinterpret_cast<int *>(qs + ldq_of(F.d));                    // [words]
+    __shared__ SelectShared S;
+    __shared__ int count;
+    const long long qi = blockIdx.x;
+    const float *q = Q + qi * F.d;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int i = threadIdx.x; i < words / 4; i += 256) reinterpret_cast<int4 *>(table)[i] = make_int4(-1, -1, -1, -1);
+    if (threadIdx.x == 0) count = 0;
+    load_query(q, F.d, qs);
+    __syncthreads();
+    for (int t = w; t < F.T; t += 8) {
+        const long long b = warp_descend(F, t, q);
+        const long long lo = (b * F.n) >> F.L;
+        const int c = (int)((((b + 1) * F.n) >> F.L) - lo);
+        const int32_t *src = F.perm + (size_t)t * F.n + lo;
+        for (int i0 = 0; i0 < c; i0 += 128) {
+            int id[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) id[u] = i0 + lane + 32 * u < c ? __ldg(src + i0 + lane + 32 * u) : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool fresh = id[u] >= 0 && seen_first<false>(table, words, id[u]);
+                __syncwarp();
+                const unsigned bl = __ballot_sync(FULL, fresh);
+                int at = 0;
+                if (lane == 0 && bl) at = atomicAdd(&count, __popc(bl));
+                at = __shfl_sync(FULL, at, 0);
+                if (fresh) kq[at + __popc(bl & lt)] = (unsigned)id[u];
+            }
+        }
+    }
+    __syncthreads();
+    const int C = count;
+    for (int j0 = w * G; j0 < C; j0 += 8 * G) {
+        int rid[G];
+        float dd[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) rid[g] = (int)(unsigned)kq[min(j0 + g, C - 1)];
+        __syncwarp();
+        warp_dist_g<PREC, NC, G>(F, qs, rid, dd);
+        unsigned long long key = KEY_NONE;
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if (lane == g) key = make_key(dd[g], rid[g]);
+        if (lane < G && j0 + lane < C) kq[j0 + lane] = key;
+    }
+    __syncthreads();
+    const int kn = select_keys<256, SEL_BUF / 256>(kq, C, keep, a, S);
+    if (PREC != P_F32) {
+        for (int j = threadIdx.x; j < kn; j += 256) S.sid[j] = (int)(unsigned)(a[j] & 0xffffffffu);
+        __syncthreads();
+        rescore_f32<NCF>(F, qs, S.sid, kn, a);
+        sort_distinct(a, kn);
+    }
+    write_topk(a, kn, k, ids + qi * k, dists + qi * k);
+    if (threadIdx.x == 0 && ncand_out) ncand_out[qi] = C;
+}
+
+// The batch in the order of the leaves it reaches in tree 0 (their first ORDER_BITS levels): one CTA,
+// a counting sort over the leaves in shared memory.  Queries of one leaf come in no particular order.
+constexpr int ORDER_BITS = 14;
+
+__global__ void __launch_bounds__(1024) k_list_order(Leaves V, int L, long long m, int *order) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int *bin = reinterpret_cast<int *>(smem_raw);  // [2^min(L, ORDER_BITS)]
+    __shared__ int wsum[32];
+    const int drop = max(0, L - ORDER_BITS), nb = 1 << (L - drop);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    auto leaf0 = [&](long long i) {
+        const unsigned b = V.plist ? V.plist[i * V.S] & ((1u << L) - 1u) : (unsigned)V.leaf[i * V.S];
+        return (int)(b >> drop);
+    };
+    for (int i = tid; i < nb; i += 1024) bin[i] = 0;
+    __syncthreads();
+    for (long long i = tid; i < m; i += 1024) atomicAdd(bin + leaf0(i), 1);
+    __syncthreads();
+    // exclusive scan: thread t owns the `per` bins from t per on
+    const int per = (nb + 1023) / 1024, beg = min(nb, tid * per), end = min(nb, beg + per);
+    int s = 0;
+    for (int i = beg; i < end; ++i) s += bin[i];
+    int inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        int x = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        wsum[lane] = x;
+    }
+    __syncthreads();
+    int run = inc - s + (w > 0 ? wsum[w - 1] : 0);
+    for (int i = beg; i < end; ++i) {
+        const int c = bin[i];
+        bin[i] = run;
+        run += c;
+    }
+    __syncthreads();
+    for (long long i = tid; i < m; i += 1024) order[atomicAdd(bin + leaf0(i), 1)] = (int)i;
 }
 
 int nc_of(int chunks) { return chunks <= 32 ? 1 : chunks <= 64 ? 2 : chunks <= 128 ? 4 : chunks <= 256 ? 8 : 0; }
@@ -336,9 +529,11 @@ int chunks_of(const gf_forest *F) {
 
 struct ListPlan {
     long long wave;     // queries per pass over the three steps
-    int S, cap, slots;  // leaves per query, list capacity, hash slots (0: bitmaps)
-    long long nwords;
-    size_t leaf, pn, okeys, order, cnt, bits, keys, total;
+    int S, cap;         // leaves per query, list capacity
+    int words;          // the shared-memory set's words (0: bitmaps in device memory)
+    bool bits_in_smem;  // a bitmap, else a hash set
+    long long nwords;   // words of a bitmap in device memory
+    size_t leaf, pn, order, cnt, bits, keys, total;
 };
 
 // Device scratch: the leaves of the whole batch and its order, then one wave's counters, bitmaps
@@ -351,18 +546,21 @@ ListPlan list_plan(const gf_forest *F, int64_t m, int leaf_budget) {
     P.S = leaf_budget > 0 ? leaf_budget : F->T;
     P.cap = (int)std::min<long long>(F->n, (long long)P.S * F->max_leaf);  // distinct ids
     const long long tot = (long long)P.S * F->max_leaf;
-    P.slots = 0;
+    P.words = 0;
+    P.bits_in_smem = false;
     if (2 * tot <= HASH_MAX) {
-        P.slots = 256;
-        while (P.slots < 2 * tot) P.slots <<= 1;
+        P.words = 256;
+        while (P.words < 2 * tot) P.words <<= 1;
+    } else if (m > FEW && F->n <= MAP_MAX) {
+        P.words = (int)((F->n + 127) / 128 * 4);
+        P.bits_in_smem = true;
     }
-    P.nwords = P.slots ? 0 : (F->n + 31) / 32;
+    P.nwords = P.words ? 0 : (F->n + 31) / 32;
     const size_t per = (size_t)P.nwords * 4 + (size_t)P.cap * 8 + 4;
     P.wave = (long long)std::max<size_t>(1, std::min<size_t>((size_t)m, WAVE_BYTES / per));
     size_t o = 0;
     P.leaf = o; o = al(o + (size_t)m * P.S * 4);
     P.pn = o; o = al(o + (leaf_budget > 0 ? (size_t)m * 4 : 0));
-    P.okeys = o; o = al(o + (m >= ORDER_MIN ? (size_t)m * 8 : 0));
     P.order = o; o = al(o + (m >= ORDER_MIN ? (size_t)m * 4 : 0));
     P.cnt = o; o = al(o + (size_t)P.wave * 4);
     P.bits = o; o = al(o + (size_t)P.wave * P.nwords * 4);  // right after the counters: zeroed with them
@@ -372,6 +570,19 @@ ListPlan list_plan(const gf_forest *F, int64_t m, int leaf_budget) {
 }
 
 size_t select_smem(const gf_forest *F, bool rerank) { return (size_t)SEL_BUF * 8 + (rerank ? (size_t)ldq_of(F->d) * 4 : 0); }
+
+template <bool BITS, bool SHORT, int NT>
+cudaError_t launch_admit(const gf_forest *F, const Leaves &V, long long q0, long long nq, const int *order,
+                         const ListPlan &P, unsigned long long *keys, int *cnt, cudaStream_t st) {
+    auto kern = k_list_admit<BITS, SHORT, NT>;
+    const size_t smem = (size_t)P.words * 4;
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)nq, NT, smem, st>>>(view_of(F), V, q0, order, P.words, P.cap, keys, cnt);
+    return cudaGetLastError();
+}
 
 template <int PREC, int NC, int G>
 cudaError_t launch_score(const gf_forest *F, const float *Q, long long q0, long long nq, const int *order,
@@ -417,6 +628,53 @@ cudaError_t launch_select(const gf_forest *F, const float *Q, long long q0, long
     return cudaGetLastError();
 }
 
+int one_words(const gf_forest *F) {
+    int words = 256;
+    while (words < 2ll * F->T * F->max_leaf) words <<= 1;
+    return words;
+}
+
+size_t one_smem(const gf_forest *F) { return (size_t)SEL_BUF * 16 + (size_t)ldq_of(F->d) * 4 + (size_t)one_words(F) * 4; }
+
+template <int PREC, int NC, int NCF>
+cudaError_t launch_one(const gf_forest *F, const float *Q, int64_t m, int k, int keep, int64_t *ids, float *dists,
+                       int *ncand_out, cudaStream_t st) {
+    auto kern = k_list_one<PREC, NC, NCF, NC == 1 ? 8 : NC == 2 ? 4 : 2>;
+    const size_t smem = one_smem(F);
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)m, 256, smem, st>>>(view_of(F), Q, k, keep, one_words(F), (long long *)ids, dists, ncand_out);
+    return cudaGetLastError();
+}
+
+template <int PREC>
+cudaError_t one_prec(const gf_forest *F, const float *Q, int64_t m, int k, int keep, int64_t *ids, float *dists,
+                     int *ncand_out, cudaStream_t st) {
+    const int nc = nc_of(chunks_of<PREC>(F)), ncf = nc_of(F->ldx / 4);
+#define GF_ONE(A, B) \
+    if (nc == A && ncf == B) return launch_one<PREC, A, B>(F, Q, m, k, keep, ids, dists, ncand_out, st);
+    if constexpr (PREC == P_F32) {
+        GF_ONE(1, 1) GF_ONE(2, 2) GF_ONE(4, 4) GF_ONE(8, 8)
+    } else {
+        GF_ONE(1, 1) GF_ONE(1, 2) GF_ONE(1, 4) GF_ONE(2, 4) GF_ONE(2, 8) GF_ONE(4, 8) GF_ONE(1, 8)
+    }
+#undef GF_ONE
+    return cudaErrorInvalidValue;
+}
+
+// One launch for the whole call: few candidates a query, rows of at most 4 KB, no reflections, little
+// to score in all, and either little for one CTA (its rows come at some 50 GB/s) or about a CTA an SM.
+// Microseconds a call, one launch / the staged steps: 640 candidates of 1 KB, m = 10: 23 / 32, 304:
+// 29 / 46, 1000: 68 / 95; 640 of 3840 bytes, m = 10: 56 / 32, 100: 56 / 54, 304: 70 / 97, 1000: 257 / 254;
+// 160 of 512 bytes, m = 100: 20 / 33, 1000: 25 / 50 (host time of the call: about 19).
+bool one_launch(const gf_forest *F, int64_t m, int32_t precision, const QueryExtra &x) {
+    if (x.leaf_budget > 0 || F->U || F->cand_cap > SEL_BUF || nc_of(F->ldx / 4) == 0 || m * F->cand_cap > ONE_MAX) return false;
+    const int chunks = precision == GF_FP32 ? chunks_of<P_F32>(F) : precision == GF_BF16_RERANK ? chunks_of<P_BF16>(F) : chunks_of<P_FP8>(F);
+    return (int64_t)F->cand_cap * chunks * 16 <= ONE_BYTES || m >= F->num_sms;
+}
+
 }  // namespace
 
 bool gf_list_usable(const gf_forest *F, int64_t m, int32_t k, int32_t precision, int32_t R, const QueryExtra &x) {
@@ -433,6 +691,16 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     *ran = false;
     const bool prio = x.leaf_budget > 0, rerank = precision != GF_FP32;
     const int keep = rerank ? R : k;
+    if (one_launch(F, m, precision, x)) {
+        *ran = true;
+        cudaError_t e = gf_record(x, 0, st);
+        if (e == cudaSuccess)
+            e = precision == GF_FP32 ? one_prec<P_F32>(F, Q, m, k, keep, ids, dists, x.ncand_out, st)
+                : precision == GF_BF16_RERANK ? one_prec<P_BF16>(F, Q, m, k, keep, ids, dists, x.ncand_out, st)
+                                              : one_prec<P_FP8>(F, Q, m, k, keep, ids, dists, x.ncand_out, st);
+        if (e == cudaSuccess) e = gf_record(x, 1, st);
+        return e == cudaSuccess ? GF_OK : gf_cuda_fail(e, "k_list_one launch");
+    }
     const ListPlan P = list_plan(F, m, x.leaf_budget);
     char *ws = nullptr;
     if (gf_scratch_alloc((void **)&ws, P.total, st) != cudaSuccess) {
@@ -466,22 +734,25 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     V.S = P.S;
     int *order = nullptr;
     if (m >= ORDER_MIN && x.order != GF_ORDER_GIVEN) {
-        unsigned long long *okeys = (unsigned long long *)(ws + P.okeys);
         order = (int *)(ws + P.order);
-        k_list_order_keys<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(V, F->L, m, okeys);
-        if ((e = gf_sort_order(m, okeys, order, st)) != cudaSuccess) return fail(e, "query order");
+        const size_t os = (size_t)4 << std::min(F->L, ORDER_BITS);
+        if (os > 40 * 1024 && (e = cudaFuncSetAttribute(k_list_order, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os)) != cudaSuccess)
+            return fail(e, "cudaFuncSetAttribute(k_list_order)");
+        k_list_order<<<1, 1024, os, st>>>(V, F->L, m, order);
+        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "k_list_order launch");
     }
     const int segs = (F->max_leaf + SEG - 1) / SEG;
+    const bool shortl = F->max_leaf <= 64;
     const int ncf = nc_of(F->ldx / 4);
     if ((e = gf_record(x, 0, st)) != cudaSuccess) return fail(e, "cudaEventRecord");
     for (long long q0 = 0; q0 < m; q0 += P.wave) {
         const long long nq = std::min<long long>(P.wave, m - q0);
-        if (P.slots) {
-            const size_t hs = (size_t)P.slots * 4;
-            if (hs > 40 * 1024 && (e = cudaFuncSetAttribute(k_list_admit_hash, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                            (int)hs)) != cudaSuccess)
-                return fail(e, "cudaFuncSetAttribute(k_list_admit_hash)");
-            k_list_admit_hash<<<(unsigned)nq, 256, hs, st>>>(view_of(F), V, q0, order, P.slots, P.cap, keys, cnt);
+        if (P.words) {
+            e = P.bits_in_smem ? (shortl ? launch_admit<true, true, 1024>(F, V, q0, nq, order, P, keys, cnt, st)
+                                         : launch_admit<true, false, 1024>(F, V, q0, nq, order, P, keys, cnt, st))
+                               : (shortl ? launch_admit<false, true, 256>(F, V, q0, nq, order, P, keys, cnt, st)
+                                         : launch_admit<false, false, 256>(F, V, q0, nq, order, P, keys, cnt, st));
+            if (e != cudaSuccess) return fail(e, "k_list_admit launch");
         } else {
             // the counters and the bitmaps lie side by side
             if ((e = cudaMemsetAsync(cnt, 0, P.bits - P.cnt + (size_t)nq * P.nwords * 4, st)) != cudaSuccess)

@@ -874,11 +874,7 @@ int gf_launch_query(const gf_forest *F, const float *Q, int64_t m, int32_t k, in
         return gf_launch_leaf(F, Q, m, k, precision, R, x.order, x.leaf_budget, st, ids, dists, x.workspace,
                               x.workspace_bytes, x.events, ctas_per_sm);
     }
-    // The staged path for everything but the smallest calls: there its launches cost more than the
-    // sort kernel's serial steps (100 queries of 160 candidates: 27.8 us against 18.8 us; 27 queries of
-    // 3136: 40 us against 164 us).
-    const bool few = x.leaf_budget == 0 && F->cand_cap <= 512 && m * F->cand_cap <= 65536 && !x.ncand_out;
-    if (x.algo == GF_ALGO_AUTO && !x.shaped && !few && gf_list_usable(F, m, k, precision, R, x)) {
+    if (x.algo == GF_ALGO_AUTO && !x.shaped && gf_list_usable(F, m, k, precision, R, x)) {
         bool ran = false;
         const int r = gf_launch_list(F, Q, m, k, precision, R, st, ids, dists, x, &ran);
         if (r || ran) return r;

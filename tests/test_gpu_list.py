@@ -37,6 +37,7 @@ SHAPES = [
     (3, 1, 1, 1, 1, 1), (500, 7, 3, 1, 9, 4), (1000, 33, 2, 1000, 5, 128), (4096, 128, 8, 1024, 3, 10),
     (4097, 130, 8, 1025, 2, 10), (8200, 96, 2, 4200, 1, 100), (20_000, 65, 16, 700, 40, 10),
     (3000, 1030, 6, 50, 600, 7), (6000, 257, 12, 30, 1, 1), (30_000, 24, 40, 500, 130, 17),
+    (2_000_000, 4, 10, 100, 1100, 5), (2_000_000, 4, 20, 1000, 30, 5),  # bitmaps past shared memory, L = 15
 ]
 
 
