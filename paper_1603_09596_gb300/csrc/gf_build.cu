@@ -18,6 +18,13 @@
 //      go left.  The h-th key is found by an 8-pass radix select; v = x_s of that key (+inf when
 //      the right child is empty, which only leaf_size 1 can produce);
 //   4. the stable partition.
+// The split dimension needs the t largest variances only, so step 1 runs twice (per-node scope, points
+// as they are): first for every dimension in 16-bit fixed point, with exact integer sums and a proven
+// bound on the rounding (k_qsum, k_cand); then, in the arithmetic above, for the few dimensions that
+// the bounds leave a place among the t largest (k_exact), which gives the same choice.  The integer
+// sums are exact, so a right child's are its parent's minus its sibling's, and half of the points are
+// read at most levels; at the root all trees hold the same points, and one of them is summed.  A
+// node whose bounds leave more than CAND_MAX dimensions goes through the full-precision kernels.
 // Levels whose nodes hold more than SMALL points use chunked kernels over all nodes of the level
 // (the variance partial sums of the chunks are added in a fixed order, so the build is
 // deterministic); deeper levels use one CTA per node that keeps the node's keys in shared memory.
@@ -294,6 +301,325 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
     }
 }
 
+// ---------------------------------------------------------------- variance bounds in fixed point
+//
+// Coordinate j of every point as q = rint((x - mid_j) / s_j), 16 bits, s_j = range_j / 65000.  Rounding
+// moves a coordinate by at most QERR s_j (half a step, plus the float32 rounding of x - mid_j and of
+// the product, under 0.01 of a step at |q| <= 32,500), so over a node of c points the square root of
+// the sum of squared deviations moves by at most QERR sqrt(c) s_j (triangle inequality), which bounds
+// the variance on both sides.  A level's sums read 2 bytes a coordinate instead of 4 and cost a few
+// integer instructions instead of some 26 of compensated float32: 500,000 x 960, T = 32, a level took
+// 15.4 ms of compensated sums (1.0e12 coordinates/s, bound by those instructions) and takes 2.1 ms of
+// k_qsum over half the points (7.4 TB/s of rows: HBM) and 0.8 ms of k_exact; the build with its bf16
+// copy and the export 174.8 -> 49.6 ms.
+constexpr int CAND_MAX = 64;       // dimensions listed per node; -1: more, the node is summed in full
+constexpr float QERR = 0.52f;
+constexpr float QSTEPS = 65000.f;  // s_j = range_j / QSTEPS
+constexpr int QCHUNK = 2048;       // points a CTA sums
+constexpr long long QSUM_BYTES = 1ll << 30;  // sums kept for a level's nodes (and its parents')
+
+__device__ __forceinline__ unsigned range_bits(float f) {
+    const unsigned u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+// rng[j], rng[d + j]: smallest and largest value of dimension j, as ordered bits (preset ~0, 0)
+__global__ void __launch_bounds__(256) k_range(const float *__restrict__ x, long long n, int d, int ldx, int rows, unsigned *rng) {
+    const int j = blockIdx.y * 256 + threadIdx.x;
+    if (j >= d) return;
+    const long long r0 = (long long)blockIdx.x * rows, r1 = min(n, r0 + rows);
+    float lo = __int_as_float(0x7f800000), hi = -lo;
+#pragma unroll 8
+    for (long long r = r0; r < r1; ++r) {
+        const float v = __ldg(x + r * ldx + j);
+        lo = fminf(lo, v);
+        hi = fmaxf(hi, v);
+    }
+    atomicMin(rng + j, range_bits(lo));
+    atomicMax(rng + d + j, range_bits(hi));
+}
+
+// qdim[j] = (mid, 1 / s, s); s = 0: a constant dimension; s < 0: a range outside [1e-30, 1e30], whose
+// variance is left unknown (q = 0)
+__global__ void k_qdim(const unsigned *__restrict__ rng, int d, float4 *qdim) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= d) return;
+    const float lo = from_ordered(rng[j]), hi = from_ordered(rng[d + j]);
+    const float range = hi - lo;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (range != 0.f) {
+        if (range >= 1e-30f && range <= 1e30f) q = make_float4(lo + 0.5f * range, QSTEPS / range, range / QSTEPS, 0.f);
+        else q.z = -1.f;
+    }
+    qdim[j] = q;
+}
+
+// xq[i][j], rows padded with zeros to ldq = round_up(d, 8); a thread makes eight values
+__global__ void __launch_bounds__(256) k_quant(const float *__restrict__ x, long long n, int d, int ldx, int ldq,
+                                               const float4 *__restrict__ qdim, short *xq) {
+    const long long total = n * (ldq / 8);
+    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
+        const long long i = g / (ldq / 8);
+        const int j0 = (int)(g - i * (ldq / 8)) * 8;
+        unsigned w[4];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = j0 + u;
+            int q = 0;
+            if (j < d) {
+                const float4 p = __ldg(qdim + j);
+                q = __float2int_rn((__ldg(x + i * ldx + j) - p.x) * p.y);
+            }
+            if (u & 1) w[u / 2] |= (unsigned)q << 16;
+            else w[u / 2] = (unsigned)q & 0xffffu;
+        }
+        *reinterpret_cast<uint4 *>(xq + i * ldq + j0) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// Which nodes of level l a k_qsum launch sums: idx counts them, seg = (tree << l) + a.
+constexpr int Q_LEFT = 0;  // the left child of every node of level l - 1
+constexpr int Q_FROM = 1;  // nodes node0 + idx
+
+__device__ __forceinline__ long long qsum_seg(int mode, int l, long long node0, long long idx) {
+    if (mode == Q_FROM) return node0 + idx;
+    return ((idx >> (l - 1)) << l) + ((idx & ((1ll << (l - 1)) - 1)) << 1);
+}
+
+// Sums of q and q^2 over a chunk of a node, per dimension, exact.  tpr threads cover a row 16 bytes
+// (eight values) each, 256 / tpr rows at a time, eight row loads in flight a thread; bound by the
+// rows it reads (one level of 500,000 x 960, T = 32: half the points, 15.4 GB, 2.05 ms).
+// sums[slot][2][d], slot = seg (Q_LEFT) or idx; several chunks a node are added with (integer, so
+// order-independent) atomics to zeroed sums.
+__global__ void __launch_bounds__(256) k_qsum(BuildParams P, int l, int mode, long long node0, int nch, int tpr,
+                                              const int *__restrict__ pin, const short *__restrict__ xq, int ldq,
+                                              long long *sums) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    long long *sh = reinterpret_cast<long long *>(smem_raw);  // [2][8 tpr]
+    const long long idx = blockIdx.x / (unsigned)nch;
+    const int ci = (int)(blockIdx.x - (unsigned)idx * (unsigned)nch);
+    const long long seg = qsum_seg(mode, l, node0, idx);
+    const NodeGeo g = geo(P, l, seg);
+    const long long beg = min(g.lo + (long long)ci * QCHUNK, g.hi), end = nch == 1 ? g.hi : min(beg + QCHUNK, g.hi);
+    const int *rows = pin + (size_t)g.tree * P.n;
+    const int col = threadIdx.x & (tpr - 1), grp = threadIdx.x / tpr, ngrp = 256 / tpr;
+    const int dbase = blockIdx.y * tpr * 8, j0 = dbase + col * 8;
+    const bool live = j0 < ldq;
+    int s1[8];
+    long long s2[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        s1[u] = 0;
+        s2[u] = 0;
+    }
+    const short *base = xq + (live ? j0 : 0);
+    auto add = [&](const uint4 v) {
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int a = (int)(w[u] << 16) >> 16, b = (int)w[u] >> 16;
+            s1[2 * u] += a;
+            s1[2 * u + 1] += b;
+            s2[2 * u] += (long long)a * a;
+            s2[2 * u + 1] += (long long)b * b;
+        }
+    };
+    constexpr int U = 8;
+    long long r = beg + grp;
+    for (; r + (U - 1) * ngrp < end; r += U * ngrp) {
+        int id[U];
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) id[u] = __ldg(rows + r + u * ngrp);
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = __ldg(reinterpret_cast<const uint4 *>(base + (size_t)id[u] * ldq));
+#pragma unroll
+        for (int u = 0; u < U; ++u) add(v[u]);
+    }
+    for (; r < end; r += ngrp) add(__ldg(reinterpret_cast<const uint4 *>(base + (size_t)__ldg(rows + r) * ldq)));
+    for (int q = ngrp - 1; q >= 0; --q) {  // the row groups add up in shared memory
+        if (grp == q) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                long long *p1 = sh + col * 8 + u, *p2 = sh + tpr * 8 + col * 8 + u;
+                *p1 = s1[u] + (q == ngrp - 1 ? 0 : *p1);
+                *p2 = s2[u] + (q == ngrp - 1 ? 0 : *p2);
+            }
+        }
+        __syncthreads();
+    }
+    long long *o = sums + (size_t)(mode == Q_FROM ? idx : seg) * 2 * P.d;
+    for (int i = threadIdx.x; i < 2 * tpr * 8; i += 256) {
+        const int h = i >= tpr * 8, j = dbase + i - h * tpr * 8;
+        if (j >= P.d) continue;
+        if (nch == 1) o[h * P.d + j] = sh[i];
+        else atomicAdd(reinterpret_cast<unsigned long long *>(o + h * P.d + j), (unsigned long long)sh[i]);
+    }
+}
+
+// Bounds of one dimension's sum of squared deviations over a node of c points, in units of
+// (c - 1) x variance, from the sums of q and q^2: evaluated in float32 with room for its rounding
+// (2^-20 of the second moment, 1e-5 of the result).
+__device__ __forceinline__ void dev_bounds(long long S1, long long S2, float c, float s, float &lo, float &hi) {
+    if (s < 0.f) {
+        lo = 0.f;
+        hi = __int_as_float(0x7f800000);
+        return;
+    }
+    const float m2 = (float)S2, m1 = (float)S1;
+    const float v = m2 - m1 * (m1 / c), e = m2 * 9.5367431640625e-7f, h = QERR * sqrtf(c);
+    const float rl = fmaxf(sqrtf(fmaxf(v - e, 0.f)) - h, 0.f) * s, rh = s == 0.f ? 0.f : (sqrtf(fmaxf(v + e, 0.f)) + h) * s;
+    lo = rl * rl * (1.f - 1e-5f);
+    hi = rh * rh * (1.f + 1e-5f);
+}
+
+// The dimensions that may be among the t of largest variance, per node: those whose upper bound
+// reaches the t-th largest of the threads' largest lower bounds (t dimensions lie at or above that).
+// derive: an odd (right) node's sums are its parent's minus its left sibling's, and are kept.
+// sums[slot], slot = blockIdx.x = seg - node0; ncand[seg] = -1 when there are more than CAND_MAX.
+__global__ void __launch_bounds__(NT) k_cand(BuildParams P, int l, long long node0, int derive,
+                                             const float4 *__restrict__ qdim, const long long *__restrict__ parent,
+                                             long long *sums, int *ncand, int *cand) {
+    __shared__ float top[NT];
+    __shared__ float tau;
+    __shared__ int count;
+    const long long seg = node0 + blockIdx.x;
+    const NodeGeo g = geo(P, l, seg);
+    const float c = (float)(g.hi - g.lo);
+    int *out = cand + seg * CAND_MAX;
+    if (g.hi - g.lo < 2) {  // every variance is 0: the first t dimensions
+        for (int r = threadIdx.x; r < P.t; r += NT) out[r] = r;
+        if (threadIdx.x == 0) ncand[seg] = P.t;
+        return;
+    }
+    long long *S = sums + (size_t)blockIdx.x * 2 * P.d;
+    const bool right = derive && (seg & 1);
+    const long long *up = right ? parent + (size_t)(l == 1 ? 0 : seg >> 1) * 2 * P.d : nullptr;
+    const long long *left = S - 2 * (size_t)P.d;
+    float best = -1.f;
+    for (int j = threadIdx.x; j < P.d; j += NT) {
+        long long S1, S2;
+        if (right) {
+            S1 = up[j] - left[j];
+            S2 = up[P.d + j] - left[P.d + j];
+            S[j] = S1;
+            S[P.d + j] = S2;
+        } else {
+            S1 = S[j];
+            S2 = S[P.d + j];
+        }
+        float lo, hi;
+        dev_bounds(S1, S2, c, qdim[j].z, lo, hi);
+        best = fmaxf(best, lo);
+    }
+    top[threadIdx.x] = best;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    int rank = 0;  // by (bound, thread)
+    for (int i = 0; i < NT; ++i) rank += top[i] > best || (top[i] == best && i < (int)threadIdx.x);
+    if (rank == P.t - 1) tau = best;
+    __syncthreads();
+    const float need = tau;
+    for (int j = threadIdx.x; j < P.d; j += NT) {
+        float lo, hi;
+        dev_bounds(S[j], S[P.d + j], c, qdim[j].z, lo, hi);
+        if (hi >= need) {
+            const int at = atomicAdd(&count, 1);
+            if (at < CAND_MAX) out[at] = j;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) ncand[seg] = count <= CAND_MAX ? count : -1;
+}
+
+// One dimension of var_accum over rows[0..cnt), cnt > 0, K the coordinate of krow: lane `lane` of
+// the warp takes dimension `dim` (negative: none).  The points come in the same order and the sums in
+// the same arithmetic, so they are var_accum's bit for bit.  Warp-wide.
+__device__ __forceinline__ void var_accum_dim(const BuildParams &P, const int *__restrict__ rows, int cnt, int krow,
+                                              int dim, double &S1, double &S2) {
+    const int lane = threadIdx.x & 31;
+    const float *xd = P.x + (dim < 0 ? 0 : dim);
+    const float K = __ldg(xd + (size_t)krow * P.ldx);
+    FF s1 = {0.f, 0.f}, s2 = {0.f, 0.f};
+    auto add = [&](float x) {
+        float dh, dl;
+        two_sum(x, -K, dh, dl);
+        const float p = dh * dh;
+        float pe = fmaf(dh, dh, -p);
+        pe = fmaf(2.f * dh, dl, pe);
+        ff_add(s1, dh, dl);
+        ff_add(s2, p, pe);
+    };
+    for (int r0 = 0; r0 < cnt; r0 += 32) {
+        const int mine = r0 + lane < cnt ? __ldg(rows + r0 + lane) : krow;
+        const int m = min(32, cnt - r0);
+        int i = 0;
+        for (; i + 8 <= m; i += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = __ldg(xd + (size_t)__shfl_sync(FULL, mine, i + u) * P.ldx);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) add(v[u]);
+        }
+        for (; i < m; ++i) add(__ldg(xd + (size_t)__shfl_sync(FULL, mine, i) * P.ldx));
+    }
+    S1 = (double)s1.hi + (double)s1.lo;
+    S2 = (double)s2.hi + (double)s2.lo;
+}
+
+// The candidate of rank `want` by (variance desc, dimension asc); lane holds candidates lane and
+// lane + 32 (d < 0: none).  Warp-wide.
+__device__ int cand_rank(const double (&v)[2], const int (&d)[2], int want) {
+    bool taken[2] = {d[0] < 0, d[1] < 0};
+    int bd = -1;
+    for (int r = 0; r <= want; ++r) {
+        double bv = -1.0;
+        bd = 0x7fffffff;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (!taken[h] && (bd == 0x7fffffff || better(v[h], d[h], bv, bd))) { bv = v[h]; bd = d[h]; }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double ov = __shfl_xor_sync(FULL, bv, o);
+            const int od = __shfl_xor_sync(FULL, bd, o);
+            if (od != 0x7fffffff && (bd == 0x7fffffff || better(ov, od, bv, bd))) { bv = ov; bd = od; }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) taken[h] = taken[h] || d[h] == bd;
+    }
+    return bd;
+}
+
+__device__ __forceinline__ int draw_rank(const BuildParams &P, unsigned long long tk, int j) {
+    return (int)(sm64_at(tk, (unsigned long long)j + 1ull) % (unsigned long long)P.t);
+}
+
+// The exact variances of a node's listed dimensions, a warp per node (nodes of at most SMALL points),
+// and the node's split dimension.
+__global__ void __launch_bounds__(NT) k_exact(BuildParams P, int l, long long nseg, const int *__restrict__ pin,
+                                              const int *__restrict__ ncand, const int *__restrict__ cand, int *seg_s) {
+    const long long seg = ((long long)blockIdx.x * NT + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (seg >= nseg) return;
+    const int nc = ncand[seg];
+    if (nc < 0) return;
+    const NodeGeo g = geo(P, l, seg);
+    const int *rows = pin + (size_t)g.tree * P.n + g.lo;
+    const int cnt = (int)(g.hi - g.lo);
+    double v[2] = {0.0, 0.0};
+    int d[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        d[h] = lane + 32 * h < nc ? cand[seg * CAND_MAX + lane + 32 * h] : -1;
+        if (32 * h < nc && cnt > 0) {
+            double S1, S2;
+            var_accum_dim(P, rows, cnt, rows[0], d[h], S1, S2);
+            v[h] = var_of(S1, S2, cnt);
+        }
+    }
+    const int s = cand_rank(v, d, draw_rank(P, tree_key(P, g.tree), g.j));
+    if (lane == 0) seg_s[seg] = s;
+}
+
 // ---------------------------------------------------------------- small levels: CTA per node
 
 struct SmallSmem {
@@ -309,7 +635,9 @@ struct SmallSmem {
     unsigned long long pref;
 };
 
+// seg_s: the split dimensions already chosen (null: none), except for nodes of ncand < 0
 __global__ void __launch_bounds__(NT) k_level_small(BuildParams P, int l, const int *__restrict__ pin,
+                                                    const int *__restrict__ seg_s, const int *__restrict__ ncand,
                                                     int *pout) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem &S = *reinterpret_cast<SmallSmem *>(smem_raw);
@@ -321,6 +649,8 @@ __global__ void __launch_bounds__(NT) k_level_small(BuildParams P, int l, const 
     // 1-2: split dimension
     if (P.global_scope && l > 0) {
         if (threadIdx.x == 0) S.s = pick_dim(P, tk, g.j, P.D);
+    } else if (seg_s && ncand[blockIdx.x] >= 0) {
+        if (threadIdx.x == 0) S.s = seg_s[blockIdx.x];
     } else {
         if (threadIdx.x == 0) S.have = 0;
         for (int dbase = 0; dbase < P.d; dbase += DB) {
@@ -371,10 +701,60 @@ __device__ __forceinline__ ChunkGeo chunk_geo(const BuildParams &P, int l, int n
     return q;
 }
 
+// The exact partial sums of a node's listed dimensions, a warp per chunk: xpart[chunk][2][CAND_MAX].
+__global__ void __launch_bounds__(NT) k_exact_chunk(BuildParams P, int l, int nch, long long nchunks, const int *__restrict__ pin,
+                                                    const int *__restrict__ ncand, const int *__restrict__ cand, double *xpart) {
+    const long long c = ((long long)blockIdx.x * NT + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (c >= nchunks) return;
+    const ChunkGeo q = chunk_geo(P, l, nch, c);
+    const int nc = ncand[q.seg], cnt = (int)(q.end - q.beg);
+    const int *seq = pin + (size_t)q.g.tree * P.n;
+    for (int h = 0; 32 * h < nc; ++h) {
+        const int dim = lane + 32 * h < nc ? cand[q.seg * CAND_MAX + lane + 32 * h] : -1;
+        double S1 = 0.0, S2 = 0.0;
+        if (cnt > 0) var_accum_dim(P, seq + q.beg, cnt, seq[q.g.lo], dim, S1, S2);
+        double *o = xpart + (size_t)c * 2 * CAND_MAX + 32 * h + lane;
+        o[0] = S1;
+        o[CAND_MAX] = S2;
+    }
+}
+
+// Adds a node's chunk sums in chunk order, ranks its listed dimensions and picks the split dimension:
+// a warp per node.  Level 0: tree 0's list and sums serve every tree.
+__global__ void __launch_bounds__(NT) k_exact_pick(BuildParams P, int l, int nch, long long nseg, const int *__restrict__ ncand,
+                                                   const int *__restrict__ cand, const double *__restrict__ xpart, int *seg_s) {
+    const long long seg = ((long long)blockIdx.x * NT + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (seg >= nseg) return;
+    const NodeGeo g = geo(P, l, seg);
+    const long long from = l == 0 ? 0 : seg;
+    const int nc = ncand[from];
+    if (nc < 0) return;
+    double v[2] = {0.0, 0.0};
+    int d[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        d[h] = lane + 32 * h < nc ? cand[from * CAND_MAX + lane + 32 * h] : -1;
+        double S1 = 0.0, S2 = 0.0;
+        if (d[h] >= 0)
+            for (int ci = 0; ci < nch; ++ci) {
+                const double *p = xpart + ((size_t)from * nch + ci) * 2 * CAND_MAX + 32 * h + lane;
+                S1 += p[0];
+                S2 += p[CAND_MAX];
+            }
+        v[h] = var_of(S1, S2, g.hi - g.lo);
+    }
+    const int s = cand_rank(v, d, draw_rank(P, tree_key(P, g.tree), g.j));
+    if (lane == 0) seg_s[seg] = s;
+}
+
 // variance partial sums of one chunk: part[c][0..d) = S1, part[c][d..2d) = S2
+// (skip: the nodes whose split dimension is chosen already, ncand >= 0; level 0: tree 0's entry)
 __global__ void __launch_bounds__(NT) k_var_partial(BuildParams P, int l, int nch, const int *__restrict__ pin,
-                                                    double *part) {
+                                                    const int *__restrict__ skip, double *part) {
     const ChunkGeo q = chunk_geo(P, l, nch, blockIdx.x);
+    if (skip && skip[l == 0 ? 0 : q.seg] >= 0) return;
     const int *seq = pin + (size_t)q.g.tree * P.n;
     const int dbase = blockIdx.y * DB;
     double S1[DPT], S2[DPT];
@@ -388,12 +768,13 @@ __global__ void __launch_bounds__(NT) k_var_partial(BuildParams P, int l, int nc
 }
 
 // add a node's chunk partials in chunk order, rank the dims, pick the split dimension
-__global__ void __launch_bounds__(NT) k_var_combine(BuildParams P, int l, int nch, const double *__restrict__ part,
-                                                    int *seg_s) {
+__global__ void __launch_bounds__(NT) k_var_combine(BuildParams P, int l, int nch, const int *__restrict__ skip,
+                                                    const double *__restrict__ part, int *seg_s) {
     __shared__ double vblk[DB];
     __shared__ double topv[TMAX];
     __shared__ int topi[TMAX];
     __shared__ int have;
+    if (skip && skip[l == 0 ? 0 : blockIdx.x] >= 0) return;
     const NodeGeo g = geo(P, l, blockIdx.x);
     const long long cnt = g.hi - g.lo;
     if (threadIdx.x == 0) have = 0;
@@ -635,7 +1016,81 @@ __global__ void k_iota(int *perm, long long n, int T) {
 struct DevBuf {
     void *p = nullptr;
     ~DevBuf() { cudaFree(p); }
+    // memory the build can do without: false (and no error left behind) if there is none
+    bool spare(size_t bytes) {
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return true;
+        cudaGetLastError();
+        p = nullptr;
+        return false;
+    }
 };
+
+// Scratch of the fixed-point pass (k_qsum and after); without it the build takes the full-precision
+// sums of every dimension.
+struct QuantScratch {
+    DevBuf rng, qdim, xq, sums[2], ncand, cand, segs, xpart;
+    int ldq = 0, tpr = 8;
+    long long cap = 0;      // nodes each sums buffer holds
+    bool on = false;
+    int have = -1;          // the level whose nodes' sums are complete in sums[have & 1]
+};
+
+// Allocates it and makes the 16-bit copy of the points.  widest: nodes of the last level.
+cudaError_t quant_prepare(QuantScratch &S, const BuildParams &P, long long widest, long long maxch, int sms, cudaStream_t st) {
+    const int d = P.d;
+    S.ldq = (d + 7) / 8 * 8;
+    while (S.tpr < 128 && S.tpr * 8 < d) S.tpr <<= 1;
+    S.cap = std::max(1ll, std::min(widest, QSUM_BYTES / (16ll * d)));
+    S.on = S.rng.spare((size_t)d * 8) && S.qdim.spare((size_t)d * 16) && S.xq.spare((size_t)P.n * S.ldq * 2) &&
+           S.sums[0].spare((size_t)S.cap * d * 16) && S.sums[1].spare((size_t)S.cap * d * 16) &&
+           S.ncand.spare((size_t)widest * 4) && S.cand.spare((size_t)widest * CAND_MAX * 4) &&
+           S.segs.spare((size_t)widest * 4) && S.xpart.spare((size_t)std::max(1ll, maxch) * 2 * CAND_MAX * 8);
+    if (!S.on) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(S.rng.p, 0xff, (size_t)d * 4, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync((unsigned *)S.rng.p + d, 0, (size_t)d * 4, st);
+    if (e != cudaSuccess) return e;
+    const int rows = 256;
+    k_range<<<dim3((unsigned)((P.n + rows - 1) / rows), (d + 255) / 256), 256, 0, st>>>(P.x, P.n, d, P.ldx, rows, (unsigned *)S.rng.p);
+    k_qdim<<<(d + 255) / 256, 256, 0, st>>>((const unsigned *)S.rng.p, d, (float4 *)S.qdim.p);
+    k_quant<<<sms * 16, 256, 0, st>>>(P.x, P.n, d, P.ldx, S.ldq, (const float4 *)S.qdim.p, (short *)S.xq.p);
+    return cudaGetLastError();
+}
+
+// The candidate dimensions of every node of level l (level 0: of the points, once).
+cudaError_t quant_level(QuantScratch &S, const BuildParams &P, int l, const int *seq, cudaStream_t st) {
+    const long long nseg = l == 0 ? 1 : (long long)P.T << l;
+    const long long cm = (P.n + (1ll << l) - 1) >> l;
+    const int nch = (int)((cm + QCHUNK - 1) / QCHUNK);
+    const int dblocks = (S.ldq + S.tpr * 8 - 1) / (S.tpr * 8);
+    const size_t smem = (size_t)2 * S.tpr * 8 * 8;
+    long long *sums = (long long *)S.sums[l & 1].p, *parent = (long long *)S.sums[(l & 1) ^ 1].p;
+    auto qsum = [&](int mode, long long node0, long long nodes, long long slots) {
+        cudaError_t e = nch > 1 ? cudaMemsetAsync(sums, 0, (size_t)slots * P.d * 16, st) : cudaSuccess;
+        if (e != cudaSuccess) return e;
+        k_qsum<<<dim3((unsigned)(nodes * nch), dblocks), 256, smem, st>>>(P, l, mode, node0, nch, S.tpr, seq,
+                                                                          (const short *)S.xq.p, S.ldq, sums);
+        return cudaGetLastError();
+    };
+    auto pick = [&](long long node0, long long nodes, int derive) {
+        k_cand<<<(unsigned)nodes, NT, 0, st>>>(P, l, node0, derive, (const float4 *)S.qdim.p, parent, sums, (int *)S.ncand.p,
+                                               (int *)S.cand.p);
+        return cudaGetLastError();
+    };
+    cudaError_t e = cudaSuccess;
+    if (l > 0 && S.have == l - 1 && nseg <= S.cap) {
+        // left children summed, right ones derived (both kinds write their sums before any child reads
+        // them: the left ones in the first launch)
+        if ((e = qsum(Q_LEFT, 0, nseg / 2, nseg)) == cudaSuccess) e = pick(0, nseg, 1);
+        S.have = l;
+        return e;
+    }
+    for (long long n0 = 0; n0 < nseg && e == cudaSuccess; n0 += S.cap) {
+        const long long nodes = std::min(S.cap, nseg - n0);
+        if ((e = qsum(Q_FROM, n0, nodes, nodes)) == cudaSuccess) e = pick(n0, nodes, 0);
+    }
+    if (nseg <= S.cap) S.have = l;
+    return e;
+}
 
 }  // namespace
 
@@ -695,6 +1150,10 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
     if (small_max > (size_t)smem_optin) return gf_fail(GF_EUNSUPPORTED, "build needs %zu B shared memory", small_max);
     GF_CUDA_TRY(cudaFuncSetAttribute(k_level_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_max));
 
+    QuantScratch S;
+    if (!F->U && !P.global_scope && L > 0) GF_CUDA_TRY(quant_prepare(S, P, (long long)T << (L - 1), maxch, F->num_sms, st));
+    const int *chosen = S.on ? (const int *)S.ncand.p : nullptr;  // >= 0: the node's split dimension is chosen below
+
     const int ndb = (F->d + DB - 1) / DB;
     for (int l = 0; l < L; ++l) {
         GfRange level_range("gf_build: level");
@@ -702,7 +1161,14 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
         const long long nseg = (long long)T << l;
         if (cm <= SMALL) {
             const size_t smem = sizeof(SmallSmem) + (size_t)cm * 8;
-            k_level_small<<<(unsigned)nseg, NT, smem, st>>>(P, l, bufA, bufB);
+            // (level 0 of a small set: every tree does its own root)
+            const bool sel = S.on && l > 0;
+            if (sel) {
+                GF_CUDA_TRY(quant_level(S, P, l, bufA, st));
+                k_exact<<<(unsigned)((nseg * 32 + NT - 1) / NT), NT, 0, st>>>(P, l, nseg, bufA, chosen, (const int *)S.cand.p,
+                                                                              (int *)S.segs.p);
+            }
+            k_level_small<<<(unsigned)nseg, NT, smem, st>>>(P, l, bufA, sel ? (const int *)S.segs.p : nullptr, chosen, bufB);
             GF_CUDA_TRY(cudaGetLastError());
         } else {
             const int nch = (int)((cm + CHUNK - 1) / CHUNK);
@@ -712,8 +1178,16 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
             unsigned *gh = (unsigned *)ghist.p;
             const unsigned gseg = (unsigned)((nseg + 255) / 256);
             if (!P.global_scope || l == 0) {
-                k_var_partial<<<dim3((unsigned)nchunks, ndb), NT, 0, st>>>(P, l, nch, bufA, (double *)part.p);
-                k_var_combine<<<(unsigned)nseg, NT, 0, st>>>(P, l, nch, (const double *)part.p, seg_s);
+                if (S.on) {
+                    GF_CUDA_TRY(quant_level(S, P, l, bufA, st));
+                    const long long own = l == 0 ? nch : nchunks;  // level 0: tree 0's chunks serve all
+                    k_exact_chunk<<<(unsigned)((own * 32 + NT - 1) / NT), NT, 0, st>>>(
+                        P, l, nch, own, bufA, chosen, (const int *)S.cand.p, (double *)S.xpart.p);
+                    k_exact_pick<<<(unsigned)((nseg * 32 + NT - 1) / NT), NT, 0, st>>>(
+                        P, l, nch, nseg, chosen, (const int *)S.cand.p, (const double *)S.xpart.p, seg_s);
+                }
+                k_var_partial<<<dim3((unsigned)nchunks, ndb), NT, 0, st>>>(P, l, nch, bufA, chosen, (double *)part.p);
+                k_var_combine<<<(unsigned)nseg, NT, 0, st>>>(P, l, nch, chosen, (const double *)part.p, seg_s);
             } else {
                 k_pick_global<<<gseg, 256, 0, st>>>(P, l, nseg, seg_s);
             }
