@@ -31,8 +31,8 @@
 //      their own) and set tau_q; every later chunk lowers it with its own R-th best (atomicMin).
 //      Nothing in the union's R best is lost: such a key lies below tau_q and among the R best of
 //      its leaf;
-//   5. merge (k_leaf_merge): per query the keys of its S lists at or below its final bound are
-//      de-duplicated by id, the R best screened ids are rescored in float32 (direct form, the same
+//   5. merge (k_leaf_merge): per query the R best ids of its S lists are found (every id once, at its
+//      best key), a screen's are rescored in float32 (direct form, the same
 //      code as the other kernels' rerank) and the k nearest are written in (distance, id) order.
 // Results are those of the screened search of the other kernels: the screen ranks the query's
 // candidate union, its R best are rescored exactly.  Screen scores near the shortlist boundary can
@@ -1044,97 +1044,142 @@ __global__ void k_qsplit8(const float *__restrict__ Q, long long m, int d, int l
 
 // ---------------------------------------------------------------- merge + rerank
 
-// Per query: the keys of its S lists of R at or below its final bound tau_q (every key of the
-// union's R best is) -> distinct ids -> the R best -> (screened keys: float32 rerank) -> k nearest.
-// One CTA per query at a time.
+// Per query: the R best distinct ids of its S lists of R keys -> (screened keys: float32 rerank) -> k
+// nearest.  One CTA per query at a time.
+//
+// The lists hold S R keys (8192 at the most) at or below the bounds their chunks knew, the same id in
+// many of them; the R best ids are a few dozen keys and their copies.  The keys are dealt to the
+// threads, and the R-th smallest of the threads' smallest keys of different ids bounds the R-th best
+// id from above.  The keys at or below that go into a hash set by id that keeps each id's smallest
+// key.  Should more than MERGE_IDS ids lie below the bound, the R-th smallest key held (of as many
+// different ids) is a lower one, and the keys are gathered again.  The lists are read twice (the second
+// time from L2) and nothing is sorted but the few keys left: 10^4 queries of 8192 keys took 5.26 ms
+// with all keys below tau_q sorted twice in shared memory (1024 keys each and R = 32: 0.82 ms).
+constexpr int MERGE_NT = 256;
+constexpr int MERGE_SLOTS = 2048;  // of the hash set
+constexpr int MERGE_IDS = 1024;    // ids it takes
+
+size_t merge_smem(const gf_forest *F, int rerank) {
+    return (size_t)MERGE_SLOTS * 12 + (size_t)MERGE_IDS * 8 + (rerank ? (size_t)ldq_of(F->d) * 4 : 0);
+}
+
 template <int NCF>
-__global__ void __launch_bounds__(128) k_leaf_merge(ForestView F, const float *__restrict__ Q, long long m, int k,
-                                                    int R, int S, int rerank,
-                                                    const unsigned long long *__restrict__ part,
-                                                    const unsigned long long *__restrict__ tau, long long *ids,
-                                                    float *dists) {
+__global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const float *__restrict__ Q, long long m, int k,
+                                                            int R, int S, int rerank,
+                                                            const unsigned long long *__restrict__ part,
+                                                            const unsigned long long *__restrict__ tau, long long *ids,
+                                                            float *dists) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int TR = S * R;
-    int Pmax = 2;
-    while (Pmax < TR) Pmax <<= 1;
-    unsigned long long *a = reinterpret_cast<unsigned long long *>(smem_raw);
-    float *qs = reinterpret_cast<float *>(a + Pmax);
-    int *sid = reinterpret_cast<int *>(qs + ldq_of(F.d));
-    unsigned char *dup = reinterpret_cast<unsigned char *>(sid + R);  // [Pmax]
-    __shared__ int nshort, nkeep;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
+    unsigned long long *hkey = reinterpret_cast<unsigned long long *>(smem_raw);  // [MERGE_SLOTS]
+    unsigned long long *a = hkey + MERGE_SLOTS;                                   // [MERGE_IDS]
+    int *hid = reinterpret_cast<int *>(a + MERGE_IDS);                            // [MERGE_SLOTS]
+    float *qs = reinterpret_cast<float *>(hid + MERGE_SLOTS);                     // [ldq], rerank only
+    __shared__ int sid[R_MAX];
+    __shared__ unsigned long long sbound;
+    __shared__ int nheld, nids;
+    const int TR = S * R, tid = threadIdx.x;
     for (long long qi = blockIdx.x; qi < m; qi += gridDim.x) {
-        const unsigned long long tq = tau[qi];
-        if (threadIdx.x == 0) {
-            nshort = 0;
-            nkeep = 0;
-        }
-        __syncthreads();
-        // the keys that can still be among the R best, as (id, score): the copies of an id
-        // come together, its best score first.  Eight loads in flight a thread; a warp appends its
-        // keepers with one atomic.
         const unsigned long long *pq = part + qi * TR;
-        for (int base = 0; base < TR; base += blockDim.x * 8) {
+        const unsigned long long tq = tau[qi];
+        // (an id outside [0, n) is a list no scoring CTA wrote: its launch gave up a wait)
+        auto usable = [&](unsigned long long key, unsigned long long bound) {
+            return key != KEY_NONE && key <= bound && (key & 0xffffffffull) < (unsigned long long)F.n;
+        };
+        unsigned long long mn = KEY_NONE;
+        for (int base = 0; base < TR; base += MERGE_NT * 8) {
             unsigned long long kv[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const int i = base + u * blockDim.x + threadIdx.x;
-                kv[u] = i < TR ? __ldcs(pq + i) : KEY_NONE;
+                const int i = base + u * MERGE_NT + tid;
+                kv[u] = i < TR ? __ldcg(pq + i) : KEY_NONE;
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const unsigned long long key = kv[u];
-                // (an id outside [0, n) is a list no scoring CTA wrote: its launch gave up a wait)
-                const bool keep = key != KEY_NONE && key <= tq && (key & 0xffffffffull) < (unsigned long long)F.n;
-                const unsigned bal = __ballot_sync(FULL, keep);
-                if (bal) {
-                    int at = 0;
-                    if (lane == 0) at = atomicAdd(&nkeep, __popc(bal));
-                    at = __shfl_sync(FULL, at, 0);
-                    if (keep) a[at + __popc(bal & lt)] = (key << 32) | (key >> 32);
-                }
-            }
-        }
-        __syncthreads();
-        const int n = nkeep;
-        int P = 2;
-        while (P < n) P <<= 1;
-        for (int i = n + threadIdx.x; i < P; i += blockDim.x) a[i] = KEY_NONE;
-        block_sort<unsigned long long>(a, P);
-        // every id once, with its best score; back to (score, id) for the second sort
-        for (int i = threadIdx.x; i < P; i += blockDim.x) dup[i] = i > 0 && (a[i] >> 32) == (a[i - 1] >> 32);
-        __syncthreads();
-        for (int i = threadIdx.x; i < P; i += blockDim.x) {
-            const unsigned long long v = a[i];
-            a[i] = dup[i] ? KEY_NONE : ((v << 32) | (v >> 32));
-        }
-        block_sort<unsigned long long>(a, P);
-        for (int i = threadIdx.x; i < R && i < P; i += blockDim.x) {
-            if (a[i] != KEY_NONE) {
-                sid[i] = (int)(unsigned)(a[i] & 0xffffffffu);
-                atomicAdd(&nshort, 1);
-            }
+            for (int u = 0; u < 8; ++u)
+                if (kv[u] < mn && usable(kv[u], tq)) mn = kv[u];
         }
         if (rerank) load_query(Q + qi * F.d, F.d, qs);
+        // the smallest keys of different ids: drop a thread's if another thread has the id at a smaller key
+        hkey[tid] = mn;
+        if (tid == 0) sbound = tq;
         __syncthreads();
-        const int C = nshort;  // the valid keys are a prefix of the sorted list
-        if (rerank) {
-            // the shortlist's ids are in sid: the keys' buffer is free for the float32 scores
-            rescore_f32<NCF>(F, qs, sid, C, a);
-            sort_keys(a, C);
-            write_topk(a, C, k, ids + qi * k, dists + qi * k);
-        } else {  // the keys are float32 distances already, in order
-            write_topk(a, C, k, ids + qi * k, dists + qi * k);
+        bool copy = mn == KEY_NONE;
+        for (int j = 0; j < MERGE_NT; ++j) {
+            const unsigned long long o = hkey[j];
+            copy |= (unsigned)o == (unsigned)mn && (o < mn || (o == mn && j < tid));
         }
+        a[tid] = copy ? KEY_NONE : mn;
+        __syncthreads();
+        int rank = 0;
+        for (int j = 0; j < MERGE_NT; ++j) rank += a[j] < mn;
+        if (!copy && rank == R - 1) sbound = mn;
+        __syncthreads();
+        int n = 0;
+        for (unsigned long long bound = sbound;;) {
+            for (int i = tid; i < MERGE_SLOTS; i += MERGE_NT) {
+                hid[i] = -1;
+                hkey[i] = KEY_NONE;
+            }
+            if (tid == 0) {
+                nheld = 0;
+                nids = 0;
+            }
+            __syncthreads();
+            for (int base = 0; base < TR; base += MERGE_NT * 8) {
+                unsigned long long kv[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int i = base + u * MERGE_NT + tid;
+                    kv[u] = i < TR ? __ldcg(pq + i) : KEY_NONE;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (!usable(kv[u], bound)) continue;
+                    const int id = (int)(unsigned)kv[u];
+                    unsigned h = ((unsigned)id * 2654435769u) >> 21;  // the top 11 bits: MERGE_SLOTS slots
+                    // at most MERGE_IDS + MERGE_NT slots are ever taken, so the probe ends
+                    for (;;) {
+                        int at = *reinterpret_cast<volatile int *>(hid + h);
+                        if (at == -1) {
+                            if (*reinterpret_cast<volatile int *>(&nids) > MERGE_IDS) break;  // full: a lower bound comes
+                            at = atomicCAS(hid + h, -1, id);
+                            if (at == -1) {
+                                atomicAdd(&nids, 1);
+                                at = id;
+                            }
+                        }
+                        if (at == id) {
+                            atomicMin(hkey + h, kv[u]);
+                            break;
+                        }
+                        h = (h + 1) & (MERGE_SLOTS - 1);
+                    }
+                }
+            }
+            __syncthreads();
+            const bool full = nids > MERGE_IDS;
+            for (int i = tid; i < MERGE_SLOTS; i += MERGE_NT) {
+                if (hid[i] >= 0) {
+                    const int at = atomicAdd(&nheld, 1);
+                    if (at < MERGE_IDS) a[at] = hkey[i];
+                }
+            }
+            __syncthreads();
+            n = min(nheld, MERGE_IDS);
+            sort_distinct(a, n);
+            if (!full) break;
+            bound = a[R - 1];
+            __syncthreads();
+        }
+        const int C = min(R, n);
+        if (rerank) {
+            for (int i = tid; i < C; i += MERGE_NT) sid[i] = (int)(unsigned)(a[i] & 0xffffffffu);
+            __syncthreads();
+            rescore_f32<NCF>(F, qs, sid, C, a);
+            sort_distinct(a, C);
+        }  // else the keys are float32 distances already, in order
+        write_topk(a, C, k, ids + qi * k, dists + qi * k);
         __syncthreads();
     }
-}
-
-size_t merge_smem(const gf_forest *F, int S, int R) {
-    int P = 2;
-    while (P < S * R) P <<= 1;
-    return (size_t)P * 8 + (size_t)ldq_of(F->d) * 4 + (size_t)R * 4 + (size_t)P;
 }
 
 // ---------------------------------------------------------------- workspace
@@ -1366,16 +1411,16 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "leaf-major scoring launch");
     if (events && (e = cudaEventRecord(events[1], st)) != cudaSuccess) return fail(e, "cudaEventRecord");
 
-    const size_t msmem = merge_smem(F, S, R);
-    const unsigned mg = (unsigned)std::min<long long>(m, (long long)F->num_sms * 16);
+    const size_t msmem = merge_smem(F, !f32);
+    const unsigned mg = (unsigned)std::min<long long>(m, (long long)F->num_sms * 64);
     const int ncf = F->ldx / 4 <= 32 ? 1 : F->ldx / 4 <= 64 ? 2 : F->ldx / 4 <= 128 ? 4 : F->ldx / 4 <= 256 ? 8 : 0;
 #define GF_MERGE(NCV)                                                                                    \
     if (ncf == NCV) {                                                                                    \
-        if (msmem > 48 * 1024 &&                                                                         \
+        if (msmem > 46 * 1024 &&                                                                         \
             (e = cudaFuncSetAttribute(k_leaf_merge<NCV>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
                                       (int)msmem)) != cudaSuccess)                                       \
             return fail(e, "cudaFuncSetAttribute(k_leaf_merge)");                                        \
-        k_leaf_merge<NCV><<<mg, 128, msmem, st>>>(view_of(F), Q, m, k, R, S, !f32, part, tau, (long long *)ids, dists); \
+        k_leaf_merge<NCV><<<mg, MERGE_NT, msmem, st>>>(view_of(F), Q, m, k, R, S, !f32, part, tau, (long long *)ids, dists); \
     }
     GF_MERGE(1) GF_MERGE(2) GF_MERGE(4) GF_MERGE(8) GF_MERGE(0)
 #undef GF_MERGE

@@ -263,24 +263,6 @@ __global__ void __launch_bounds__(256, 2) k_list_score(ForestView F, const float
 
 // ---------------------------------------------------------------- selection and rerank
 
-// Ascending sort of the distinct keys a[0..n) by counting, for every key, the smaller ones (three
-// barriers; a bitonic sort of 64 keys takes 21): up to one key a thread.  More go to the bitonic sort.
-__device__ void sort_distinct(unsigned long long *a, int n) {
-    if (n > (int)blockDim.x) {
-        sort_keys(a, n);
-        return;
-    }
-    __syncthreads();
-    const unsigned long long key = (int)threadIdx.x < n ? a[threadIdx.x] : 0ull;
-    int rank = 0;
-    if ((int)threadIdx.x < n) {
-        for (int j = 0; j < n; ++j) rank += a[j] < key;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < n) a[rank] = key;
-    __syncthreads();
-}
-
 struct SelectShared {
     unsigned hist[256];
     unsigned long long pref, bound;

@@ -158,6 +158,24 @@ __device__ void sort_keys(unsigned long long *keys, int C) {
     block_sort<unsigned long long>(keys, P);
 }
 
+// Ascending sort of the distinct keys a[0..n) by counting, for every key, the smaller ones (three
+// barriers; a bitonic sort of 64 keys takes 21): up to one key a thread.  More go to the bitonic sort.
+__device__ void sort_distinct(unsigned long long *a, int n) {
+    if (n > (int)blockDim.x) {
+        sort_keys(a, n);
+        return;
+    }
+    __syncthreads();
+    const unsigned long long key = (int)threadIdx.x < n ? a[threadIdx.x] : 0ull;
+    int rank = 0;
+    if ((int)threadIdx.x < n) {
+        for (int j = 0; j < n; ++j) rank += a[j] < key;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < n) a[rank] = key;
+    __syncthreads();
+}
+
 __device__ void write_topk(const unsigned long long *keys, int C, int k, long long *ids,
                            float *dists) {
     for (int i = threadIdx.x; i < k; i += blockDim.x) {
