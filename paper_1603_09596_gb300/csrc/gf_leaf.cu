@@ -677,158 +677,248 @@ __global__ void __maxnreg__((LeafCfg<FMT, CPS, CH>::REGS)) k_leaf_score(ForestVi
 //
 // The plain float32 search through the same regrouping: each chunk's leaf rows against its
 // queries in the direct form sum_j (q_j - x_j)^2, float32 arithmetic (packed f32x2 pairs, rounded
-// per lane as the scalar instructions), on the CUDA cores.  Row tiles of 256 rows: lane l of warp w
-// owns rows 64 w + l and 64 w + 32 + l of the tile and accumulates every query of the chunk for
-// them.  The rows stream through a two-stage cp.async ring of 32-float slabs (128 bytes per row);
-// the 16-byte chunk c of row r sits at chunk c ^ (r & 7), so a warp's 16-byte loads of 32
-// consecutive rows fall on distinct banks.  The queries' slabs sit beside them (a padded float32
-// copy of the batch) and are read by broadcast.  Keys are (distance bits, id); the per-warp lists,
-// the bound tau_q and the per-chunk merge are those of the bf16 kernel, with the k best kept per
-// (query, tree); the lists are merged in the ring's memory, idle between chunks.
+// per lane as the scalar instructions), on the CUDA cores.  A group of WPC warps works on one chunk,
+// 64 WPC rows at a time (leaves of at most 64 rows: one warp, of at most 128: two, else four; a leaf
+// of 49 rows keeps one warp of a 256-row tile busy and three idle): lane l of the group's warp w owns
+// rows 64 w + l and 64 w + 32 + l of the tile and accumulates every query of the chunk for them as a
+// packed pair of sums over the even and the odd dimensions, in ascending order.  The rows stream
+// through a cp.async ring of KS-float slabs; the 16-byte pieces of a row are placed so that a warp's
+// loads of the same piece of consecutive rows fall on distinct banks.  The queries' slabs sit beside
+// them (a padded float32 copy of the batch) and are read by broadcast.  The inner loops are compiled
+// for each even number of queries, so the loads of the next queries are scheduled among the
+// arithmetic of the last and no slots are padded to groups of four.  Keys are (distance bits, id);
+// the per-warp lists, the bound tau_q and the per-chunk merge are those of the bf16 kernel, with the k
+// best kept per (query, tree); the lists are merged in the ring's memory, idle between chunks.
+//
+// 10^4 queries, 10^5 x 960, T = 16, p = 64 (leaves of 49 rows, five queries each): one chunk a CTA
+// 6.1 ms a step, one a warp 2.3 ms; 10^6 x 960, T = 32, p = 1024: 33.8 -> 29.8 ms with the loops per
+// query count, one barrier a slab.  There the FMA pipe bounds it (14.9 ms of subtractions and fused
+// multiply-adds at its full rate; two warps of three wait for shared memory or for their last result).
 namespace f32k {
 constexpr int THREADS = 128;
-constexpr int CTAS_PER_SM = 3;
-constexpr int ROWS = 256;
-constexpr int KS = 32;                          // floats per slab: one 128-byte row segment
-constexpr int STAGES = 2;
-constexpr int X_BYTES = ROWS * KS * 4;          // the tile's rows of one slab
-constexpr int Q_BYTES = NQ * KS * 4;            // the chunk's queries of one slab
-constexpr int STAGE_BYTES = X_BYTES + Q_BYTES;
-constexpr int WL_BYTES = 4 * NQ * 32 * 8;       // the four warps' lists
-constexpr int SMEM = STAGES * STAGE_BYTES;
-static_assert(THREADS / 8 == NQ, "copy duty: eight threads per query row");
-static_assert(WL_BYTES <= SMEM, "the lists reuse the ring");
-__device__ __forceinline__ int swz(int r, int c) { return c ^ (r & 7); }
+
+template <int WPC>
+struct Cfg {
+    static constexpr int CTAS_PER_SM = WPC == 1 ? 2 : 3;
+    static constexpr int GROUPS = 4 / WPC;               // chunks a CTA works on
+    static constexpr int GT = 32 * WPC;                  // threads of a group
+    static constexpr int ROWS = 64 * WPC;                // rows of a tile
+    static constexpr int KS = 32;                        // floats per slab: one 128-byte row segment
+    static constexpr int STAGES = 2;
+    static constexpr int PIECES = KS / 4;                // 16-byte pieces of a row's slab
+    static constexpr int X_BYTES = ROWS * KS * 4;
+    static constexpr int Q_BYTES = NQ * KS * 4;
+    static constexpr int STAGE_BYTES = X_BYTES + Q_BYTES;
+    static constexpr int GROUP_BYTES = STAGES * STAGE_BYTES;
+    static constexpr int SMEM = GROUPS * GROUP_BYTES;
+    static constexpr int STEP = GT / PIECES;             // rows a copy pass of the group covers
+    static_assert(WPC * NQ * 32 * 8 <= GROUP_BYTES, "the lists reuse the ring");
+    static_assert(CTAS_PER_SM * (SMEM + 1024) <= 228 * 1024, "shared memory of the CTAs of one SM");
+    // where piece c of row r sits among the pieces of its row
+    static __device__ __forceinline__ int swz(int r, int c) { return c ^ (r & 7); }
+    static __device__ __forceinline__ void sync(int group) {
+        if (WPC == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(GT) : "memory");
+    }
+};
 }  // namespace f32k
 
-__global__ void __launch_bounds__(f32k::THREADS, f32k::CTAS_PER_SM) k_leaf_f32(ForestView F, LeafArgs A) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned long long *wl = reinterpret_cast<unsigned long long *>(smem_raw);  // between chunks only
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int item_lo = *A.item_lo, item_hi = *A.item_hi;
-    const int NS = (F.d + f32k::KS - 1) / f32k::KS;  // slabs per row tile
-    const int R = A.R;
-    int RL = 1;
-    while (RL < R) RL <<= 1;
-    const int cc = tid & 7, cr = tid >> 3;  // copy duty: 16-byte chunk cc of rows cr + 16 i, query cr
-    const uint32_t sbase = smem_u32(smem_raw);
-    for (int w = item_lo + blockIdx.x; w < item_hi; w += gridDim.x) {
-        int t, rows, q0pos, nq;
-        long long lo;
-        chunk_of(F, A, w, t, lo, rows, q0pos, nq);
-        const int ng = (nq + 3) >> 2;  // groups of four queries
-        const int qid_c = cr < nq ? A.qlist[q0pos + cr] / A.S : -1;
-        const int my_qid = lane < nq ? A.qlist[q0pos + lane] / A.S : 0;
-        const unsigned long long my_tau = lane < nq ? __ldcg(A.tau + my_qid) : KEY_NONE;
-        unsigned long long lst[NQ];
+struct F32Chunk {
+    const int *perm;  // the leaf's point ids
+    int rows, nq, q0pos;
+};
+
+// A slab of the lane's two rows (xs0, xs1: their 16-byte pieces, placed by swz) against the first NV
+// queries: acc[row][query] += the squared differences, in ascending dimension order.  Where every warp
+// has a chunk of its own they run different NV at a time, and the loops together have to stay in the
+// instruction cache: rolled over the pieces, and nothing but the loop compiled per NV (with the whole
+// chunk compiled per NV the warps waited for instructions five cycles of every six).
+template <int WPC, int NV>
+__device__ __forceinline__ void f32_slab(const unsigned char *xs0, const unsigned char *xs1, int r0, const float *qs,
+                                         unsigned long long (&acc)[2][NQ]) {
+    using C = f32k::Cfg<WPC>;
+#pragma unroll(WPC == 1 ? 1 : 2)
+    for (int c4 = 0; c4 < C::PIECES; ++c4) {
+        // four floats as two packed pairs (low half first): no repacking; rows 32 apart swizzle alike
+        const int at = C::swz(r0, c4) << 4;
+        const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(xs0 + at);
+        const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(xs1 + at);
 #pragma unroll
-        for (int j = 0; j < NQ; ++j) lst[j] = KEY_NONE;
-        const int *perm_leaf = F.perm + (size_t)t * F.n + lo;
-        const int MT = (rows + f32k::ROWS - 1) / f32k::ROWS;
-        for (int mt = 0; mt < MT; ++mt) {
-            int ids[f32k::ROWS / 16];
-#pragma unroll
-            for (int i = 0; i < f32k::ROWS / 16; ++i) {
-                const int r = mt * f32k::ROWS + cr + 16 * i;
-                ids[i] = r < rows ? __ldg(perm_leaf + r) : -1;
-            }
-            auto load_slab = [&](int sl, int stg) {
-                const int col = sl * f32k::KS + cc * 4;
-                const int nbytes = max(0, min(16, (F.d - col) * 4));
-                const uint32_t xs = sbase + stg * f32k::STAGE_BYTES;
-#pragma unroll
-                for (int i = 0; i < f32k::ROWS / 16; ++i) {
-                    const int r = cr + 16 * i;
-                    const bool live = ids[i] >= 0 && nbytes > 0;
-                    const float *src = live ? F.x + (size_t)ids[i] * F.ldx + col : F.x;
-                    cp_async16(xs + r * (f32k::KS * 4) + (f32k::swz(r, cc) << 4), src, live ? nbytes : 0);
-                }
-                {
-                    const bool live = qid_c >= 0 && nbytes > 0;
-                    const float *src = live ? A.qf + (size_t)qid_c * F.ldx + col : A.qf;
-                    cp_async16(xs + f32k::X_BYTES + cr * f32k::KS * 4 + cc * 16, src, live ? nbytes : 0);
-                }
-                cp_async_commit();
-            };
-            unsigned long long acc[2][NQ];  // packed (even, odd) partial sums per (row, query)
-#pragma unroll
-            for (int a = 0; a < 2; ++a)
-#pragma unroll
-                for (int j = 0; j < NQ; ++j) acc[a][j] = 0ull;
-            // double buffer: slab sl + 1 is requested while slab sl is scored
-            load_slab(0, 0);
-            for (int sl = 0; sl < NS; ++sl) {
-                if (sl + 1 < NS) load_slab(sl + 1, (sl + 1) & 1);
-                else cp_async_commit();
-                cp_async_wait<1>();
-                __syncthreads();
-                const unsigned char *xs = smem_raw + (sl & 1) * f32k::STAGE_BYTES;
-                const float *qs = reinterpret_cast<const float *>(xs + f32k::X_BYTES);
-                const int r0 = 64 * warp + lane, r1 = r0 + 32;
-#pragma unroll 2
-                for (int c4 = 0; c4 < f32k::KS / 4; ++c4) {
-                    // four floats as two packed pairs (low half first): no repacking
-                    const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(xs + r0 * (f32k::KS * 4) + (f32k::swz(r0, c4) << 4));
-                    const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(xs + r1 * (f32k::KS * 4) + (f32k::swz(r1, c4) << 4));
-                    const unsigned long long a01 = x0.x, a23 = x0.y, b01 = x1.x, b23 = x1.y;
-#pragma unroll
-                    for (int g = 0; g < NQ / 4; ++g) {
-                        if (g < ng) {
-#pragma unroll
-                            for (int jj = 0; jj < 4; ++jj) {
-                                const int j = 4 * g + jj;
-                                const ulonglong2 qv = *reinterpret_cast<const ulonglong2 *>(qs + j * f32k::KS + c4 * 4);
-                                const unsigned long long q01 = qv.x, q23 = qv.y;
-                                unsigned long long e = sub2(q01, a01);
-                                acc[0][j] = fma2(e, e, acc[0][j]);
-                                e = sub2(q23, a23);
-                                acc[0][j] = fma2(e, e, acc[0][j]);
-                                e = sub2(q01, b01);
-                                acc[1][j] = fma2(e, e, acc[1][j]);
-                                e = sub2(q23, b23);
-                                acc[1][j] = fma2(e, e, acc[1][j]);
-                            }
-                        }
-                    }
-                }
-                __syncthreads();  // the stage is refilled two slabs later
-            }
-            // the tile's distances: the warp's 64 rows against every query of the chunk
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const int r = mt * f32k::ROWS + 64 * warp + 32 * a + lane;
-                const bool valid = r < rows;
-                const int id = valid ? __ldg(perm_leaf + r) : 0;
-#pragma unroll
-                for (int j = 0; j < NQ; ++j) {
-                    if (j < nq) {
-                        const float2 s = upk(acc[a][j]);
-                        const unsigned long long key = valid ? make_key(s.x + s.y, id) : KEY_NONE;
-                        const unsigned long long thr =
-                            umin64(__shfl_sync(FULL, lst[j], R - 1), __shfl_sync(FULL, my_tau, j));
-                        const unsigned bl = __ballot_sync(FULL, key < thr);
-                        if (bl) lst[j] = list_add(lst[j], key, bl, R, RL);
-                    }
-                }
-            }
+        for (int j = 0; j < NV; ++j) {
+            const ulonglong2 qv = *reinterpret_cast<const ulonglong2 *>(qs + j * C::KS + c4 * 4);
+            unsigned long long e = sub2(qv.x, x0.x);
+            acc[0][j] = fma2(e, e, acc[0][j]);
+            e = sub2(qv.y, x0.y);
+            acc[0][j] = fma2(e, e, acc[0][j]);
+            e = sub2(qv.x, x1.x);
+            acc[1][j] = fma2(e, e, acc[1][j]);
+            e = sub2(qv.y, x1.y);
+            acc[1][j] = fma2(e, e, acc[1][j]);
         }
-        // the chunk is done: merge the four warps' lists; each query's R best of this leaf
-#pragma unroll
-        for (int j = 0; j < NQ; ++j)
-            if (j < nq) wl[(warp * NQ + j) * 32 + lane] = lst[j];
-        __syncthreads();
-        for (int j = warp; j < nq; j += 4) {
-            unsigned long long a = wl[(0 * NQ + j) * 32 + lane], b = wl[(1 * NQ + j) * 32 + lane];
-            unsigned long long c = wl[(2 * NQ + j) * 32 + lane], d = wl[(3 * NQ + j) * 32 + lane];
-            if (lane >= RL) a = b = c = d = KEY_NONE;
-            const unsigned long long best = warp_merge_top(warp_merge_top(a, b, RL), warp_merge_top(c, d, RL), RL);
-            const int pr = A.qlist[q0pos + j];  // q S + slot
-            if (lane < R) A.part[(size_t)pr * R + lane] = best;
-            const unsigned long long kth = __shfl_sync(FULL, best, R - 1);
-            if (lane == 0 && kth != KEY_NONE) atomicMin(A.tau + pr / A.S, kth);
-        }
-        __syncthreads();  // the lists are rewritten by the next chunk
     }
+}
+
+// One chunk by its group.
+template <int WPC>
+__device__ __forceinline__ void f32_chunk(const ForestView &F, const LeafArgs &A, const F32Chunk &ch, unsigned char *ring,
+                                          int group, int gt, int RL) {
+    using C = f32k::Cfg<WPC>;
+    constexpr int KS = C::KS, NV = NQ;
+    const int warp = gt >> 5, lane = gt & 31;  // within the group
+    const int nq = ch.nq, R = A.R;
+    const int NS = (F.d + KS - 1) / KS;  // slabs per row tile
+    const int cc = gt % C::PIECES, cr = gt / C::PIECES;  // copy duty: piece cc of rows cr + STEP i
+    const uint32_t sbase = smem_u32(ring);
+    int qid_c[NQ / C::STEP > 0 ? NQ / C::STEP : 1];      // ... and of queries cr + STEP i
+#pragma unroll
+    for (int i = 0; i < (NQ / C::STEP > 0 ? NQ / C::STEP : 1); ++i) {
+        const int j = cr + C::STEP * i;
+        qid_c[i] = j < nq ? A.qlist[ch.q0pos + j] / A.S : -1;
+    }
+    const int my_qid = lane < nq ? A.qlist[ch.q0pos + lane] / A.S : 0;
+    const unsigned long long my_tau = lane < nq ? __ldcg(A.tau + my_qid) : KEY_NONE;
+    unsigned long long lst[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) lst[j] = KEY_NONE;
+    const int MT = (ch.rows + C::ROWS - 1) / C::ROWS;
+    for (int mt = 0; mt < MT; ++mt) {
+        int ids[C::ROWS / C::STEP];
+#pragma unroll
+        for (int i = 0; i < C::ROWS / C::STEP; ++i) {
+            const int r = mt * C::ROWS + cr + C::STEP * i;
+            ids[i] = r < ch.rows ? __ldg(ch.perm + r) : -1;
+        }
+        auto load_slab = [&](int sl) {
+            const int col = sl * KS + cc * 4;
+            const int nbytes = max(0, min(16, (F.d - col) * 4));
+            const uint32_t xs = sbase + (sl % C::STAGES) * C::STAGE_BYTES;
+#pragma unroll
+            for (int i = 0; i < C::ROWS / C::STEP; ++i) {
+                const int r = cr + C::STEP * i;
+                const bool live = ids[i] >= 0 && nbytes > 0;
+                const float *src = live ? F.x + (size_t)ids[i] * F.ldx + col : F.x;
+                cp_async16(xs + r * (KS * 4) + (C::swz(r, cc) << 4), src, live ? nbytes : 0);
+            }
+#pragma unroll
+            for (int i = 0; i < (NQ / C::STEP > 0 ? NQ / C::STEP : 1); ++i) {
+                const int j = cr + C::STEP * i;
+                if (C::STEP > NQ && j >= NQ) break;
+                const bool live = qid_c[i] >= 0 && nbytes > 0;
+                const float *src = live ? A.qf + (size_t)qid_c[i] * F.ldx + col : A.qf;
+                cp_async16(xs + C::X_BYTES + j * (KS * 4) + cc * 16, src, live ? nbytes : 0);
+            }
+        };
+        unsigned long long acc[2][NV];  // packed (even, odd) partial sums per (row, query)
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int j = 0; j < NV; ++j) acc[a][j] = 0ull;
+        // the ring: STAGES - 1 slabs are requested ahead of the one that is scored
+#pragma unroll
+        for (int sl = 0; sl < C::STAGES - 1; ++sl) {
+            if (sl < NS) load_slab(sl);
+            cp_async_commit();
+        }
+        for (int sl = 0; sl < NS; ++sl) {
+            cp_async_wait<C::STAGES - 2>();
+            C::sync(group);  // the slab has arrived, and slab sl - 1 is scored: its place is free
+            if (sl + C::STAGES - 1 < NS) load_slab(sl + C::STAGES - 1);
+            cp_async_commit();
+            const unsigned char *xs = ring + (sl % C::STAGES) * C::STAGE_BYTES;
+            const float *qs = reinterpret_cast<const float *>(xs + C::X_BYTES);
+            const int r0 = 64 * warp + lane;
+            const unsigned char *xs0 = xs + r0 * (KS * 4), *xs1 = xs0 + 32 * KS * 4;
+            switch ((nq + 1) >> 1) {
+                case 1: f32_slab<WPC, 2>(xs0, xs1, r0, qs, acc); break;
+                case 2: f32_slab<WPC, 4>(xs0, xs1, r0, qs, acc); break;
+                case 3: f32_slab<WPC, 6>(xs0, xs1, r0, qs, acc); break;
+                case 4: f32_slab<WPC, 8>(xs0, xs1, r0, qs, acc); break;
+                case 5: f32_slab<WPC, 10>(xs0, xs1, r0, qs, acc); break;
+                case 6: f32_slab<WPC, 12>(xs0, xs1, r0, qs, acc); break;
+                case 7: f32_slab<WPC, 14>(xs0, xs1, r0, qs, acc); break;
+                default: f32_slab<WPC, 16>(xs0, xs1, r0, qs, acc); break;
+            }
+        }
+        C::sync(group);  // the ring is refilled by the next tile
+        // the tile's distances: the warp's 64 rows against every query of the chunk
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int r = mt * C::ROWS + 64 * warp + 32 * a + lane;
+            const bool valid = r < ch.rows;
+            const int id = valid ? __ldg(ch.perm + r) : 0;
+#pragma unroll
+            for (int j = 0; j < NV; ++j) {
+                if (j < nq) {
+                    const float2 s = upk(acc[a][j]);
+                    const unsigned long long key = valid ? make_key(s.x + s.y, id) : KEY_NONE;
+                    const unsigned long long thr = umin64(__shfl_sync(FULL, lst[j], R - 1), __shfl_sync(FULL, my_tau, j));
+                    const unsigned bl = __ballot_sync(FULL, key < thr);
+                    if (bl) lst[j] = list_add(lst[j], key, bl, R, RL);
+                }
+            }
+        }
+    }
+    // the chunk is done: merge the warps' lists; each query's R best of this leaf
+    unsigned long long *wl = reinterpret_cast<unsigned long long *>(ring);
+    if (WPC > 1) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j)
+            if (j < nq) wl[(warp * NQ + j) * 32 + lane] = lst[j];
+        C::sync(group);
+    }
+    auto finish = [&](int j, unsigned long long best) {
+        const int pr = A.qlist[ch.q0pos + j];  // q S + slot
+        if (lane < R) A.part[(size_t)pr * R + lane] = best;
+        const unsigned long long kth = __shfl_sync(FULL, best, R - 1);
+        if (lane == 0 && kth != KEY_NONE) atomicMin(A.tau + pr / A.S, kth);
+    };
+    if (WPC == 1) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j)
+            if (j < nq) finish(j, lane < RL ? lst[j] : KEY_NONE);
+    } else {
+        for (int j = warp; j < nq; j += WPC) {
+            unsigned long long a = wl[(0 * NQ + j) * 32 + lane], b = wl[(1 * NQ + j) * 32 + lane];
+            unsigned long long c = WPC == 4 ? wl[(2 * NQ + j) * 32 + lane] : KEY_NONE;
+            unsigned long long d = WPC == 4 ? wl[(3 * NQ + j) * 32 + lane] : KEY_NONE;
+            if (lane >= RL) a = b = c = d = KEY_NONE;
+            finish(j, WPC == 4 ? warp_merge_top(warp_merge_top(a, b, RL), warp_merge_top(c, d, RL), RL)
+                               : warp_merge_top(a, b, RL));
+        }
+        C::sync(group);  // the lists are read before the next chunk's rows come
+    }
+}
+
+template <int WPC>
+__global__ void __launch_bounds__(f32k::THREADS, f32k::Cfg<WPC>::CTAS_PER_SM) k_leaf_f32(ForestView F, LeafArgs A) {
+    using C = f32k::Cfg<WPC>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int group = threadIdx.x / C::GT, gt = threadIdx.x % C::GT;
+    unsigned char *ring = smem_raw + group * C::GROUP_BYTES;
+    const int item_lo = *A.item_lo, item_hi = *A.item_hi;
+    int RL = 1;
+    while (RL < A.R) RL <<= 1;
+    for (int w = item_lo + blockIdx.x * C::GROUPS + group; w < item_hi; w += gridDim.x * C::GROUPS) {
+        int t;
+        long long lo;
+        F32Chunk ch;
+        chunk_of(F, A, w, t, lo, ch.rows, ch.q0pos, ch.nq);
+        ch.perm = F.perm + (size_t)t * F.n + lo;
+        f32_chunk<WPC>(F, A, ch, ring, group, gt, RL);
+    }
+}
+
+// warps per chunk for a forest's leaves, and its launch
+int f32_wpc(const gf_forest *F) { return F->max_leaf <= 64 ? 1 : F->max_leaf <= 128 ? 2 : 4; }
+
+template <int WPC>
+cudaError_t f32_attr() {
+    return cudaFuncSetAttribute(k_leaf_f32<WPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, f32k::Cfg<WPC>::SMEM);
+}
+
+template <int WPC>
+void f32_launch(const gf_forest *F, const LeafArgs &A, cudaStream_t st) {
+    k_leaf_f32<WPC><<<F->num_sms * f32k::Cfg<WPC>::CTAS_PER_SM, f32k::THREADS, f32k::Cfg<WPC>::SMEM, st>>>(view_of(F), A);
 }
 
 // q -> a float32 copy with rows padded to ldx (16-byte aligned rows for the copies)
@@ -1381,7 +1471,8 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     const int cps = ctas_per_sm == 1 ? 1 : 2;
     // two chunks share a row tile when no leaf has more than 64 rows (half a tile)
     const int ch = ((F->n + (1ll << F->L) - 1) >> F->L) <= BM / 2 ? 2 : 1;
-    e = f32 ? cudaFuncSetAttribute(k_leaf_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, f32k::SMEM)
+    const int wpc = f32_wpc(F);
+    e = f32 ? (wpc == 1 ? f32_attr<1>() : wpc == 2 ? f32_attr<2>() : f32_attr<4>())
         : f8 ? score_attr<LF_FP8>(cps, ch) : score_attr<LF_BF16>(cps, ch);
     if (e != cudaSuccess) return fail(e, "cudaFuncSetAttribute(leaf-major scoring)");
     LeafArgs A;
@@ -1404,7 +1495,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     for (int wave = 0; wave < 2; ++wave) {
         A.item_lo = wave == 0 ? koff : koff + (1 << F->L);
         A.item_hi = wave == 0 ? koff + (1 << F->L) : koff + nk;
-        if (f32) k_leaf_f32<<<F->num_sms * f32k::CTAS_PER_SM, f32k::THREADS, f32k::SMEM, st>>>(view_of(F), A);
+        if (f32) wpc == 1 ? f32_launch<1>(F, A, st) : wpc == 2 ? f32_launch<2>(F, A, st) : f32_launch<4>(F, A, st);
         else if (f8) score_launch<LF_FP8>(cps, ch, F, A, st);
         else score_launch<LF_BF16>(cps, ch, F, A, st);
     }
