@@ -1,12 +1,12 @@
 // gf_list.cu -- the staged per-query path: the search of gf_query.cu (Alg. 2; Eq. 1; Sec. 2.3;
 // Sec. 3 "Distance computation") cut into launches, so that the work of a query is not bound to one
 // CTA:
-//   1. the leaves of every (query, tree): gf_descend, or one warp per pair (k_list_descend), or the
-//      priority search's list;
+//   1. the leaves of every (query, tree): gf_descend, or one warp per pair (k_list_descend, or the
+//      admission's own warps), or the priority search's list;
 //   2. admit: the points of a query's leaves are written to its candidate list once each (the "seen"
 //      array of Sec. 2.3): through a hash set or a bitmap over the point ids in shared memory, one CTA
-//      a query; for a few queries of many candidates, or too many points for that, through a bitmap in
-//      device memory, a warp per 128 positions of a leaf;
+//      a query; where the points are too many for that, through a bitmap in device memory, a warp per
+//      128 positions of a leaf;
 //   3. score (k_list_score): CTAs take blocks of rows of the lists, a warp G rows at a time;
 //   4. select (k_list_select): one CTA a query finds the `keep` smallest keys (distance, id), rescores
 //      a screen's shortlist in float32 and writes the k nearest.
@@ -17,9 +17,10 @@
 // Why: a query that is one CTA's alone reads its rows at that CTA's rate, and its descent,
 // de-duplication and sorts stand between the reads.  Here step 3 is a flat pass over all rows of the
 // batch that the whole chip shares.  Microseconds a call on one GB300, the one-CTA kernels -> this:
-//   1 query, 10^6 x 960, T = 32, p = 1024, bf16 (10.9k rows)         856 -> 33   (streaming)
-//   199 queries, 5 10^5 x 960, T = 32, p = 512, bf16 (5.6k rows)     779 -> 328  (streaming)
-//   27 queries, 5 10^4 x 512, T = 16, p = 256, float32               165 -> 39   (sort)
+//   1 query, 10^6 x 960, T = 32, p = 1024, bf16 (10.9k rows)         950 -> 29   (streaming)
+//   199 queries, 5 10^5 x 960, T = 32, p = 512, bf16 (5.6k rows)     742 -> 324  (streaming)
+//   27 queries, 5 10^4 x 512, T = 16, p = 256, float32               160 -> 30   (sort)
+//   2000 queries, 2 10^5 x 10^4, T = 24, p = 32, E4M3               3173 -> 2238 (sort)
 //   10^4 queries, 10^6 x 960, T = 32, p = 64, bf16 (1.24k rows)     8798 -> 3037 (sort)
 //   5003 queries, 7 10^5 x 101, T = 32, p = 64, float32              890 -> 419  (sort)
 // The scoring step is bound by the row loads: 9.8 TB/s of rows at 10^4 queries (most from L2, whose
@@ -38,7 +39,6 @@ constexpr int GROUPS = 256;        // groups of keys whose minima bound the keep
 constexpr int SEL_BUF = 1024;      // keys at or below that bound the selection holds
 constexpr int HASH_MAX = 16384;    // slots of the shared-memory hash set (at least twice the ids)
 constexpr int MAP_MAX = 1800000;   // points whose bitmap fits shared memory (225,000 bytes)
-constexpr int FEW = 16;            // batches up to here spread a query's admission over many CTAs
 constexpr int SEG = 128;           // positions of a leaf a warp admits at once (four a lane)
 constexpr int ONE_MAX = 640000;    // candidates of a call that runs in one launch,
 constexpr int ONE_BYTES = 768 << 10;  // and bytes of a query's rows there, with fewer queries than SMs
@@ -51,6 +51,11 @@ struct Leaves {
     const int *pn;
     int S;  // leaves per query
 };
+
+// The steps' launches overlap (programmatic dependent launch): a kernel may start once every CTA of the
+// one before it has begun, prepares what does not depend on it, and waits here for its end.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // slot s of query q: its first position in perm and its length (0 when the query has fewer leaves)
 __device__ __forceinline__ int leaf_of(const ForestView &F, const Leaves &V, long long q, int s, long long &base) {
@@ -69,41 +74,57 @@ __device__ __forceinline__ int leaf_of(const ForestView &F, const Leaves &V, lon
     return (int)(hi - lo);
 }
 
-// The leaf of tree t that query q reaches (Eq. 1), by a whole warp: it loads the five-level subtree
-// below the current node at once (lane i: node i in breadth-first order, with the query's coordinate)
-// and walks it in the ballot of the comparisons, so a path of L nodes costs ceil(L / 5) rounds of
-// dependent loads instead of L.  For batches of a few thousand (query, tree) pairs, where the chip has
-// warps to spare and the latency of the chain is what counts.
-__device__ __forceinline__ int warp_descend(const ForestView &F, int t, const float *__restrict__ q) {
+// The leaves of trees t0 .. t0 + N - 1 (below T) that query q reaches (Eq. 1), by a whole warp: per tree
+// it loads the five-level subtree below the current node at once (lane i: node i in breadth-first
+// order, with the query's coordinate) and walks it in the ballot of the comparisons, so a path of L
+// nodes costs ceil(L / 5) rounds of dependent loads instead of L, and the trees go level in step.
+// For batches of a few thousand (query, tree) pairs, where the chip has warps to spare and the
+// latency of the chain is what counts.
+template <int N>
+__device__ __forceinline__ void warp_descend(const ForestView &F, int t0, const float *__restrict__ q, int (&leaf)[N]) {
     const int lane = threadIdx.x & 31;
-    const int2 *nodes = F.nodes + (size_t)t * F.nnodes;
     const int lv = 31 - __clz(lane + 1);  // lane's level in the subtree (lanes 0..30)
-    int j = 0;
-    while (j < F.nnodes) {
-        const long long node = (((long long)j + 1) << lv) - 1 + (lane + 1 - (1 << lv));
-        bool left = false;
-        if (lane < 31 && node < F.nnodes) {
-            const int2 nd = __ldg(nodes + node);
-            left = __ldg(q + nd.x) < __int_as_float(nd.y);
+    int j[N];
+#pragma unroll
+    for (int h = 0; h < N; ++h) j[h] = 0;
+    for (int l0 = 0; l0 < F.L; l0 += 5) {  // (the trees are perfect: every path has L nodes)
+        unsigned lefts[N];
+        int2 nd[N];
+        bool in[N];
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            const long long node = (((long long)j[h] + 1) << lv) - 1 + (lane + 1 - (1 << lv));
+            in[h] = lane < 31 && node < F.nnodes && t0 + h < F.T;
+            if (in[h]) nd[h] = __ldg(F.nodes + (size_t)(t0 + h) * F.nnodes + node);
         }
-        const unsigned lefts = __ballot_sync(FULL, left);
-        int bi = 0;
-        for (int l = 0; l < 5 && j < F.nnodes; ++l) {
-            const int side = (lefts >> bi) & 1u ? 1 : 2;
-            j = 2 * j + side;
-            bi = 2 * bi + side;
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            const bool left = in[h] && __ldg(q + nd[h].x) < __int_as_float(nd[h].y);
+            lefts[h] = __ballot_sync(FULL, left);
+        }
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            int bi = 0;
+            for (int l = l0; l < min(l0 + 5, F.L); ++l) {
+                const int side = (lefts[h] >> bi) & 1u ? 1 : 2;
+                j[h] = 2 * j[h] + side;
+                bi = 2 * bi + side;
+            }
         }
     }
-    return j - F.nnodes;
+#pragma unroll
+    for (int h = 0; h < N; ++h) leaf[h] = j[h] - F.nnodes;
 }
 
 __global__ void __launch_bounds__(128) k_list_descend(ForestView F, const float *__restrict__ Q, long long pairs,
                                                       int *leaf) {
     const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    pdl_next();
     if (g >= pairs) return;
     const long long qi = g / F.T;
-    const int b = warp_descend(F, (int)(g - qi * F.T), Q + qi * F.d);
-    if ((threadIdx.x & 31) == 0) leaf[g] = b;
+    int b[1];
+    warp_descend<1>(F, (int)(g - qi * F.T), Q + qi * F.d, b);
+    if ((threadIdx.x & 31) == 0) leaf[g] = b[0];
 }
 
 // ---------------------------------------------------------------- admission
@@ -128,17 +149,20 @@ __device__ __forceinline__ bool seen_first(int *table, int words, int id) {
 // there, written to the query's list.  BITS: a bitmap over the point ids; else a hash set (open
 // addressing, linear probing; the table has at least twice as many slots as ids, so a probe ends).
 // A warp has eight ids a lane in flight: of one leaf, or (SHORT: leaves of at most 64) of four.
-template <bool BITS, bool SHORT, int NT>
-__global__ void __launch_bounds__(NT) k_list_admit(ForestView F, Leaves V, long long q0, const int *__restrict__ order,
+// DESC: one leaf per tree, and the warps find the leaves themselves (a launch less).
+template <bool BITS, bool SHORT, int NT, bool DESC>
+__global__ void __launch_bounds__(NT) k_list_admit(ForestView F, const float *__restrict__ Q, Leaves V, long long q0, const int *__restrict__ order,
                                                    int words, int cap, unsigned long long *keys, int *cnt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int *table = reinterpret_cast<int *>(smem_raw);  // [words], a multiple of four
     __shared__ int count;
     const long long w0 = blockIdx.x;
-    const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
     const int none = BITS ? 0 : -1;
     for (int i = threadIdx.x; i < words / 4; i += NT) reinterpret_cast<int4 *>(table)[i] = make_int4(none, none, none, none);
     if (threadIdx.x == 0) count = 0;
+    pdl_wait();
+    pdl_next();
+    const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -147,11 +171,21 @@ __global__ void __launch_bounds__(NT) k_list_admit(ForestView F, Leaves V, long 
     constexpr int E = 8 / PER;          // ids a lane of each
     for (int s = w * PER; s < V.S; s += NT / 32 * PER) {
         long long base[PER];
-        int c[PER], longest = 0;
+        int c[PER], longest = 0, leaf[PER];
+        if (DESC) warp_descend<PER>(F, s, Q + qi * F.d, leaf);
 #pragma unroll
         for (int h = 0; h < PER; ++h) {
             base[h] = 0;
-            c[h] = s + h < V.S ? leaf_of(F, V, qi, s + h, base[h]) : 0;
+            c[h] = 0;
+            if (s + h < V.S) {
+                if (DESC) {
+                    const long long b = leaf[h], lo = (b * F.n) >> F.L;
+                    base[h] = (long long)(s + h) * F.n + lo;
+                    c[h] = (int)((((b + 1) * F.n) >> F.L) - lo);
+                } else {
+                    c[h] = leaf_of(F, V, qi, s + h, base[h]);
+                }
+            }
             longest = max(longest, c[h]);
         }
         for (int i0 = 0; i0 < longest; i0 += 32 * E) {
@@ -192,6 +226,7 @@ __global__ void __launch_bounds__(256) k_list_admit_bits(ForestView F, Leaves V,
     const unsigned lt = (1u << lane) - 1u;
     const long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long per = (long long)V.S * segs, w0 = g / per;
+    pdl_next();
     if (w0 >= nq) return;
     const int r = (int)(g - w0 * per), s = r / segs, p0 = (r - s * segs) * SEG;
     const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
@@ -229,6 +264,12 @@ __global__ void __launch_bounds__(256) k_list_admit_bits(ForestView F, Leaves V,
 
 // ---------------------------------------------------------------- scoring
 
+// 16-byte chunks of each of the G rows a lane has in flight when rows are longer than 4 KB: sixteen
+// loads, as for shorter rows (E4M3, d = 10^4: 1.87 ms with two chunks, 1.70 ms with four; fewer rows at
+// once read the query from shared memory more often: G = 2 2.5 ms).
+constexpr int LONG_UNR = 4;
+constexpr unsigned EARLY_GRID = 2048;  // CTAs of a scoring launch of few queries
+
 // Block `part` of B rows of query slot w0's list: ids in, keys (distance, id) out, in place.
 template <int PREC, int NC, int G>
 __global__ void __launch_bounds__(256, 2) k_list_score(ForestView F, const float *__restrict__ Q, long long q0,
@@ -237,14 +278,19 @@ __global__ void __launch_bounds__(256, 2) k_list_score(ForestView F, const float
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const long long w0 = blockIdx.x / (unsigned)parts;
     const int lo = (int)(blockIdx.x - (unsigned)w0 * (unsigned)parts) * B;
-    const int nb = min(B, cnt[w0] - lo);
-    if (nb <= 0) return;
     float *qs = reinterpret_cast<float *>(smem_raw);
     int *ids = reinterpret_cast<int *>(qs + ldq_of(F.d));
+    // few queries: the query row comes in while the admission ends
+    const bool early = !order && gridDim.x <= EARLY_GRID;
+    if (early) load_query(Q + (q0 + w0) * F.d, F.d, qs);
+    pdl_wait();
+    pdl_next();
+    const int nb = min(B, cnt[w0] - lo);
+    if (nb <= 0) return;
     const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
     unsigned long long *kq = keys + w0 * cap + lo;
     for (int j = threadIdx.x; j < nb; j += blockDim.x) ids[j] = (int)(unsigned)kq[j];
-    load_query(Q + qi * F.d, F.d, qs);
+    if (!early) load_query(Q + qi * F.d, F.d, qs);
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int j0 = w * G; j0 < nb; j0 += nw * G) {
@@ -252,7 +298,7 @@ __global__ void __launch_bounds__(256, 2) k_list_score(ForestView F, const float
         float dd[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) rid[g] = ids[min(j0 + g, nb - 1)];
-        warp_dist_g<PREC, NC, G>(F, qs, rid, dd);
+        warp_dist_g<PREC, NC, G, LONG_UNR>(F, qs, rid, dd);
         unsigned long long key = KEY_NONE;
 #pragma unroll
         for (int g = 0; g < G; ++g)
@@ -369,9 +415,12 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_list_select(ForestVie
     float *qs = reinterpret_cast<float *>(a + SEL_BUF);                        // [ldq], rerank only
     __shared__ SelectShared S;
     const long long w0 = blockIdx.x;
+    if (rerank && !order) load_query(Q + (q0 + w0) * F.d, F.d, qs);
+    pdl_wait();
+    pdl_next();
     const long long qi = order ? (long long)order[q0 + w0] : q0 + w0;
     const int C = cnt[w0];
-    if (rerank) load_query(Q + qi * F.d, F.d, qs);
+    if (rerank && order) load_query(Q + qi * F.d, F.d, qs);
     const int kn = select_keys<NT, NT == 256 ? 8 : 24>(keys + w0 * cap, C, keep, a, S);
     if (rerank) {
         for (int j = threadIdx.x; j < kn; j += NT) S.sid[j] = (int)(unsigned)(a[j] & 0xffffffffu);
@@ -405,8 +454,9 @@ __global__ void __launch_bounds__(256) k_list_one(ForestView F, const float *__r
     load_query(q, F.d, qs);
     __syncthreads();
     for (int t = w; t < F.T; t += 8) {
-        const long long b = warp_descend(F, t, q);
-        const long long lo = (b * F.n) >> F.L;
+        int leaf[1];
+        warp_descend<1>(F, t, q, leaf);
+        const long long b = leaf[0], lo = (b * F.n) >> F.L;
         const int c = (int)((((b + 1) * F.n) >> F.L) - lo);
         const int32_t *src = F.perm + (size_t)t * F.n + lo;
         for (int i0 = 0; i0 < c; i0 += 128) {
@@ -533,7 +583,7 @@ ListPlan list_plan(const gf_forest *F, int64_t m, int leaf_budget) {
     if (2 * tot <= HASH_MAX) {
         P.words = 256;
         while (P.words < 2 * tot) P.words <<= 1;
-    } else if (m > FEW && F->n <= MAP_MAX) {
+    } else if (F->n <= MAP_MAX) {
         P.words = (int)((F->n + 127) / 128 * 4);
         P.bits_in_smem = true;
     }
@@ -553,17 +603,46 @@ ListPlan list_plan(const gf_forest *F, int64_t m, int leaf_budget) {
 
 size_t select_smem(const gf_forest *F, bool rerank) { return (size_t)SEL_BUF * 8 + (rerank ? (size_t)ldq_of(F->d) * 4 : 0); }
 
-template <bool BITS, bool SHORT, int NT>
-cudaError_t launch_admit(const gf_forest *F, const Leaves &V, long long q0, long long nq, const int *order,
+// A launch that may begin while the kernel before it in the stream ends (its threads call pdl_wait).
+template <typename... KP, typename... Args>
+cudaError_t launch_after(void (*kern)(KP...), long long grid, int block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, static_cast<KP>(args)...);
+}
+
+template <bool BITS, bool SHORT, int NT, bool DESC>
+cudaError_t launch_admit_d(const gf_forest *F, const float *Q, const Leaves &V, long long q0, long long nq, const int *order,
                          const ListPlan &P, unsigned long long *keys, int *cnt, cudaStream_t st) {
-    auto kern = k_list_admit<BITS, SHORT, NT>;
+    auto kern = k_list_admit<BITS, SHORT, NT, DESC>;
     const size_t smem = (size_t)P.words * 4;
     if (smem > 40 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)nq, NT, smem, st>>>(view_of(F), V, q0, order, P.words, P.cap, keys, cnt);
-    return cudaGetLastError();
+    if (DESC) {  // the call's first launch
+        kern<<<(unsigned)nq, NT, smem, st>>>(view_of(F), Q, V, q0, order, P.words, P.cap, keys, cnt);
+        return cudaGetLastError();
+    }
+    return launch_after(kern, nq, NT, smem, st, view_of(F), Q, V, q0, order, P.words, P.cap, keys, cnt);
+}
+
+template <bool BITS, int NT>
+cudaError_t launch_admit(const gf_forest *F, const float *Q, const Leaves &V, long long q0, long long nq, const int *order,
+                         const ListPlan &P, bool desc, unsigned long long *keys, int *cnt, cudaStream_t st) {
+    if (F->max_leaf <= 64)
+        return desc ? launch_admit_d<BITS, true, NT, true>(F, Q, V, q0, nq, order, P, keys, cnt, st)
+                    : launch_admit_d<BITS, true, NT, false>(F, Q, V, q0, nq, order, P, keys, cnt, st);
+    return desc ? launch_admit_d<BITS, false, NT, true>(F, Q, V, q0, nq, order, P, keys, cnt, st)
+                : launch_admit_d<BITS, false, NT, false>(F, Q, V, q0, nq, order, P, keys, cnt, st);
 }
 
 template <int PREC, int NC, int G>
@@ -579,8 +658,7 @@ cudaError_t launch_score(const gf_forest *F, const float *Q, long long q0, long 
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)(nq * parts), 256, smem, st>>>(view_of(F), Q, q0, order, parts, B, P.cap, cnt, keys);
-    return cudaGetLastError();
+    return launch_after(kern, nq * parts, 256, smem, st, view_of(F), Q, q0, order, parts, B, P.cap, cnt, keys);
 }
 
 template <int PREC>
@@ -605,9 +683,8 @@ cudaError_t launch_select(const gf_forest *F, const float *Q, long long q0, long
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)nq, NT, smem, st>>>(view_of(F), Q, q0, k, keep, rerank, order, P.cap, cnt, keys,
-                                              (long long *)ids, dists, ncand_out);
-    return cudaGetLastError();
+    return launch_after(kern, nq, NT, smem, st, view_of(F), Q, q0, k, keep, rerank, order, P.cap, cnt, keys, (long long *)ids,
+                        dists, ncand_out);
 }
 
 int one_words(const gf_forest *F) {
@@ -650,7 +727,7 @@ cudaError_t one_prec(const gf_forest *F, const float *Q, int64_t m, int k, int k
 // to score in all, and either little for one CTA (its rows come at some 50 GB/s) or about a CTA an SM.
 // Microseconds a call, one launch / the staged steps: 640 candidates of 1 KB, m = 10: 23 / 32, 304:
 // 29 / 46, 1000: 68 / 95; 640 of 3840 bytes, m = 10: 56 / 32, 100: 56 / 54, 304: 70 / 97, 1000: 257 / 254;
-// 160 of 512 bytes, m = 100: 20 / 33, 1000: 25 / 50 (host time of the call: about 19).
+// 160 of 512 bytes, m = 100: 20 / 33, 1000: 25 / 50 (of which the host's part was about 19; now 13).
 bool one_launch(const gf_forest *F, int64_t m, int32_t precision, const QueryExtra &x) {
     if (x.leaf_budget > 0 || F->U || F->cand_cap > SEL_BUF || nc_of(F->ldx / 4) == 0 || m * F->cand_cap > ONE_MAX) return false;
     const int chunks = precision == GF_FP32 ? chunks_of<P_F32>(F) : precision == GF_BF16_RERANK ? chunks_of<P_BF16>(F) : chunks_of<P_FP8>(F);
@@ -700,7 +777,10 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     cudaError_t e = cudaSuccess;
     int r = GF_OK;
     const long long pairs = (long long)m * F->T;
-    if (prio) r = gf_launch_prio_leaves(F, Q, m, P.S, (unsigned *)leaf, pn, st);
+    // small batches: the admission's warps descend the trees
+    const bool desc = !prio && !F->U && P.words && m < ORDER_MIN && pairs <= 16384;
+    if (desc) {
+    } else if (prio) r = gf_launch_prio_leaves(F, Q, m, P.S, (unsigned *)leaf, pn, st);
     else if (pairs <= 16384 && !F->U) {
         k_list_descend<<<(unsigned)((pairs + 3) / 4), 128, 0, st>>>(view_of(F), Q, pairs, leaf);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "k_list_descend launch");
@@ -724,16 +804,15 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "k_list_order launch");
     }
     const int segs = (F->max_leaf + SEG - 1) / SEG;
-    const bool shortl = F->max_leaf <= 64;
     const int ncf = nc_of(F->ldx / 4);
     if ((e = gf_record(x, 0, st)) != cudaSuccess) return fail(e, "cudaEventRecord");
     for (long long q0 = 0; q0 < m; q0 += P.wave) {
         const long long nq = std::min<long long>(P.wave, m - q0);
         if (P.words) {
-            e = P.bits_in_smem ? (shortl ? launch_admit<true, true, 1024>(F, V, q0, nq, order, P, keys, cnt, st)
-                                         : launch_admit<true, false, 1024>(F, V, q0, nq, order, P, keys, cnt, st))
-                               : (shortl ? launch_admit<false, true, 256>(F, V, q0, nq, order, P, keys, cnt, st)
-                                         : launch_admit<false, false, 256>(F, V, q0, nq, order, P, keys, cnt, st));
+            // few queries: a whole SM's threads for each
+            e = P.bits_in_smem ? launch_admit<true, 1024>(F, Q, V, q0, nq, order, P, desc, keys, cnt, st)
+                : nq <= F->num_sms ? launch_admit<false, 1024>(F, Q, V, q0, nq, order, P, desc, keys, cnt, st)
+                                   : launch_admit<false, 256>(F, Q, V, q0, nq, order, P, desc, keys, cnt, st);
             if (e != cudaSuccess) return fail(e, "k_list_admit launch");
         } else {
             // the counters and the bitmaps lie side by side

@@ -199,8 +199,9 @@ __device__ void load_query(const float *q, int d, float *qs) {
 }
 
 // Squared distances of the query (shared memory) to G rows at once, by the whole warp; every lane
-// returns all G sums.  NC > 0: at most NC 16-byte chunks per lane; NC == 0: any row length.
-template <int PREC, int NC, int G>
+// returns all G sums.  NC > 0: at most NC 16-byte chunks per lane; NC == 0: any row length, UNR chunks
+// of every row in flight (the order of the additions does not depend on it).
+template <int PREC, int NC, int G, int UNR = 2>
 __device__ __forceinline__ void warp_dist_g(const ForestView &F, const float *qs, const int (&ids)[G],
                                             float (&d)[G]) {
     constexpr int QF4 = Prec<PREC>::QF4;
@@ -216,7 +217,7 @@ __device__ __forceinline__ void warp_dist_g(const ForestView &F, const float *qs
         acc[g] = make_float4(0.f, 0.f, 0.f, 0.f);
         sc[g] = PREC == P_FP8 ? __ldg(F.scale8 + ids[g]) : 0.f;
     }
-    constexpr int UB = NC > 0 ? NC : 2;
+    constexpr int UB = NC > 0 ? NC : UNR;
     for (int c0 = lane; c0 < nch; c0 += 32 * UB) {
         uint4 x[G][UB];
 #pragma unroll
