@@ -152,7 +152,6 @@ inline cudaError_t gf_record(const QueryExtra &x, int i, cudaStream_t st) {
 
 int gf_launch_prio_leaves(const gf_forest *F, const float *Q, int64_t m, int budget, unsigned *leaves,
                           int *nleaves, cudaStream_t st);
-size_t gf_prio_smem_bytes(int budget, int T);
 int gf_stream_workspace_bytes(const gf_forest *F, int64_t m, long long grid, bool ordered, int leaf_budget,
                               int64_t *bytes);
 // CTAs of a streaming launch of m queries with this shape (warps, ctas_per_sm 0 = occupancy limit)

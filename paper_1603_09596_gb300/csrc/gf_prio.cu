@@ -13,13 +13,20 @@
 //
 // One warp per query.  The queue is two sorted arrays in shared memory: a large one A and a small
 // one B (at most 64 entries).  A pop takes the smaller of their heads.  The entries a descent pushes
-// (at most L <= 30) are merged into B by the warp; once B holds more than 32 it is merged into A in
-// place (from the top down), so the large array moves once every few pops instead of at every one.
-// The first phase (one entry per tree and level) merges into A directly.  Entries ranked beyond the
-// number of pops still to come can never be taken and are dropped, so A never holds more than
-// `budget` entries past its head.  The order of the pops is that of a single sorted queue: every
+// (at most L <= 30, one a lane) are merged into B by the warp; once B holds more than 32 it is merged
+// into A in place (from the top down), so the large array moves once every few pops instead of at every
+// one.  The first phase (one entry per tree and level) merges into A directly.  Entries ranked beyond
+// the number of pops still to come can never be taken and are dropped, so A never holds more than
+// `budget` - T entries past its start.  The order of the pops is that of a single sorted queue: every
 // pop takes the smallest (key, tree, node) held.  The output is the list of leaves in the order
 // checked, encoded (tree << L) | leaf.
+//
+// A pop is a chain of dependent steps (head, subtree loads, walk, merge), so what counts is the length
+// of that chain and the warps an SM holds beside each other.  Merges exchange entries by shuffles and
+// ballots, and an entry's new place comes from counting, not from binary searches through shared
+// memory (six dependent loads an entry); an entry is a key of 8 bytes and a (tree, node) of 4.
+// 10^4 queries, L = 14, T = 32, 512 leaves: 5.75 ms with searches and 16-byte entries (16 warps an SM),
+// 2.71 ms now (32).
 #include "gf_internal.cuh"
 #include "gf_trace.cuh"
 
@@ -28,124 +35,138 @@
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int PRIO_WARPS = 4;  // at most this many warps (queries) per CTA
+constexpr int PRIO_WARPS = 4;   // at most this many warps (queries) per CTA
+constexpr int PQ_BCAP = 64;     // entries of the small queue array
 
-struct PQE {
-    unsigned long long key;  // bits of the float64 key |q_s - v| (>= 0)
-    int tree;
-    int node;
-};
-
-__device__ __forceinline__ bool pq_less(const PQE &a, const PQE &b) {
-    if (a.key != b.key) return a.key < b.key;
-    if (a.tree != b.tree) return a.tree < b.tree;
-    return a.node < b.node;
-}
-
+// bits of the float64 key |q_s - v| (>= 0): they order as the value does
 __device__ __forceinline__ unsigned long long pq_key(float qs, float v) {
     return (unsigned long long)__double_as_longlong(fabs((double)qs - (double)v));
 }
 
-__device__ __forceinline__ PQE pq_inf() {
-    PQE e;
-    e.key = 0x7ff0000000000000ull;  // +inf
-    e.tree = 0x7fffffff;
-    e.node = 0x7fffffff;
+// A queue entry: the key, and the place (tree << (L + 1)) | node that breaks ties by (tree, node).
+// Place: 32 bits where T 2^(L+1) <= 2^32, else 64.
+template <typename Place>
+struct PQE {
+    unsigned long long key;
+    Place at;
+};
+
+template <typename Place>
+__device__ __forceinline__ bool pq_less(const PQE<Place> &a, const PQE<Place> &b) {
+    return a.key < b.key || (a.key == b.key && a.at < b.at);
+}
+
+template <typename Place>
+__device__ __forceinline__ PQE<Place> pq_inf() {
+    PQE<Place> e;
+    e.key = ~0ull;
+    e.at = ~(Place)0;
     return e;
 }
 
-// Merge the nb (<= 32) entries of stage[] into the sorted array src[0..cnt); write the first
-// min(cnt + nb, keep) entries of the merged order to dst[]; returns their number.  Warp-wide.
-__device__ int pq_merge(const PQE *src, int cnt, PQE *stage, int nb, PQE *dst, int keep, PQE *sorted) {
+// A queue array in shared memory, keys and places apart.
+template <typename Place>
+struct PQArray {
+    unsigned long long *key;
+    Place *at;
+    __device__ __forceinline__ PQE<Place> get(int i) const {
+        PQE<Place> e;
+        e.key = key[i];
+        e.at = at[i];
+        return e;
+    }
+    __device__ __forceinline__ void set(int i, const PQE<Place> &e) const {
+        key[i] = e.key;
+        at[i] = e.at;
+    }
+    __device__ __forceinline__ PQArray from(int i) const {
+        PQArray a;
+        a.key = key + i;
+        a.at = at + i;
+        return a;
+    }
+};
+
+template <typename Place>
+__device__ __forceinline__ PQE<Place> pq_shfl(const PQE<Place> &e, int src) {
+    PQE<Place> r;
+    r.key = __shfl_sync(FULL, e.key, src);
+    r.at = __shfl_sync(FULL, e.at, src);
+    return r;
+}
+
+// Merge the nb entries held one a lane (in any order) into the sorted array b[head .. head + cnt), cnt + nb
+// <= PQ_BCAP, and leave the first min(cnt + nb, keep) of the merged order at b[0 ..); returns their number.
+// Every entry's place is the number of entries below it, counted as the new ones go round the warp.
+template <typename Place>
+__device__ int pq_insert(const PQArray<Place> &b, int head, int cnt, const PQE<Place> &mine, int nb, int keep) {
     const int lane = threadIdx.x & 31;
-    // rank of every staged entry among the staged entries (all distinct)
-    PQE mine = lane < nb ? stage[lane] : pq_inf();
-    int r = 0;
-    for (int i = 0; i < nb; ++i) r += pq_less(stage[i], mine);
-    __syncwarp();
-    if (lane < nb) sorted[r] = mine;
-    __syncwarp();
-    // staged entry r goes to r + (number of src entries below it)
-    if (lane < nb) {
-        int lo = 0, hi = cnt;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (pq_less(src[mid], mine)) lo = mid + 1;
-            else hi = mid;
-        }
-        const int pos = r + lo;
-        if (pos < keep) dst[pos] = mine;
+    const bool in0 = lane < cnt, in1 = lane + 32 < cnt;
+    const PQE<Place> b0 = in0 ? b.get(head + lane) : pq_inf<Place>(), b1 = in1 ? b.get(head + lane + 32) : pq_inf<Place>();
+    int up0 = 0, up1 = 0, pos = keep;
+    for (int i = 0; i < nb; ++i) {
+        const PQE<Place> e = pq_shfl(mine, i);
+        const bool l0 = pq_less(b0, e), l1 = pq_less(b1, e), lm = lane < nb && pq_less(mine, e);
+        up0 += !l0;
+        up1 += !l1;
+        const int below = __popc(__ballot_sync(FULL, in0 && l0)) + __popc(__ballot_sync(FULL, in1 && l1)) +
+                          __popc(__ballot_sync(FULL, lm));
+        if (lane == i) pos = below;
     }
-    // src entry j goes to j + (number of staged entries below it)
-    for (int j = lane; j < cnt; j += 32) {
-        const PQE e = src[j];
-        int lo = 0, hi = nb;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (pq_less(sorted[mid], e)) lo = mid + 1;
-            else hi = mid;
-        }
-        const int pos = j + lo;
-        if (pos < keep) dst[pos] = e;
-    }
+    __syncwarp();  // every lane has read its entries
+    if (in0 && lane + up0 < keep) b.set(lane + up0, b0);
+    if (in1 && lane + 32 + up1 < keep) b.set(lane + 32 + up1, b1);
+    if (lane < nb && pos < keep) b.set(pos, mine);
     __syncwarp();
     return min(cnt + nb, keep);
 }
 
-// Number of entries of the sorted array a[0..n) below e.  Warp lanes call it independently.
-__device__ __forceinline__ int pq_lower(const PQE *a, int n, const PQE &e) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (pq_less(a[mid], e)) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// sorted[0..nb) = the nb (<= 32) staged entries in order.  Warp-wide.
-__device__ void pq_sort_stage(const PQE *stage, int nb, PQE *sorted) {
-    const int lane = threadIdx.x & 31;
-    const PQE mine = lane < nb ? stage[lane] : pq_inf();
-    int r = 0;
-    for (int i = 0; i < nb; ++i) r += pq_less(stage[i], mine);
-    __syncwarp();
-    if (lane < nb) sorted[r] = mine;
-    __syncwarp();
-}
-
-// Merge the sorted array s[0..ns) (ns <= 64, not overlapping a) into the sorted array a[0..na) in
+// Merge the sorted array s[0..ns) (ns <= PQ_BCAP, not overlapping a) into the sorted array a[0..na) in
 // place, keeping the first min(na + ns, keep) entries of the merged order in a[]; returns their
-// number.  a[] must have room for them.  An entry of a moves up by the number of s entries below
-// it, so a is moved from the top down, 32 entries at a time, each group read before it is written.
-// Warp-wide.
-__device__ int pq_merge_into(PQE *a, int na, const PQE *s, int ns, int keep) {
+// number.  a[] must have room for them.  Entry i of s goes p_i entries of a further on (a binary search a
+// lane); an entry j of a moves up by the number of p_i <= j, so a is moved from the top down to the
+// smallest p_i, 32 entries at a time, each group read before it is written.  Warp-wide.
+template <typename Place>
+__device__ int pq_merge_into(const PQArray<Place> &a, int na, const PQArray<Place> &s, int ns, int keep) {
     const int lane = threadIdx.x & 31;
-    // the positions of s's entries in the merged order, against a as it is now
-    int ps[2];
-    PQE es[2];
+    int p[2];
+    PQE<Place> e[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int i = lane + 32 * h;
-        es[h] = i < ns ? s[i] : pq_inf();
-        ps[h] = i < ns ? i + pq_lower(a, na, es[h]) : keep;
+        e[h] = i < ns ? s.get(i) : pq_inf<Place>();
+        int lo = 0, hi = i < ns ? na : 0;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (pq_less(a.get(mid), e[h])) lo = mid + 1;
+            else hi = mid;
+        }
+        p[h] = i < ns ? lo : 0x7fffffff;
     }
-    __syncwarp();
-    for (int top = na; top > 0; top -= 32) {
-        const int j = top - 32 + lane;
-        PQE e;
-        int pos = keep;
-        if (j >= 0) {
-            e = a[j];
-            pos = j + pq_lower(s, ns, e);
+    const int first = __shfl_sync(FULL, p[0], 0);
+    for (int top = na; top > first; top -= 32) {
+        const int low = top - 32, j = low + lane;
+        PQE<Place> x = pq_inf<Place>();
+        if (j >= 0) x = a.get(j);
+        int up = __popc(__ballot_sync(FULL, p[0] < low)) + __popc(__ballot_sync(FULL, p[1] < low));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            unsigned here = __ballot_sync(FULL, p[h] >= low && p[h] < top);
+            while (here) {
+                const int src = __ffs(here) - 1;
+                here &= here - 1;
+                up += __shfl_sync(FULL, p[h], src) <= j;
+            }
         }
         __syncwarp();
-        if (j >= 0 && pos < keep) a[pos] = e;
+        if (j >= 0 && up > 0 && j + up < keep) a.set(j + up, x);
         __syncwarp();
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (ps[h] < keep) a[ps[h]] = es[h];
+    for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h;
+        if (i < ns && i + p[h] < keep) a.set(i + p[h], e[h]);
+    }
     __syncwarp();
     return min(na + ns, keep);
 }
@@ -154,25 +175,27 @@ __device__ __forceinline__ unsigned leaf_code(int tree, int leaf, int L) {
     return ((unsigned)tree << L) | (unsigned)leaf;
 }
 
-constexpr int PQ_BCAP = 64;  // entries of each small queue array
+// entries of the large array: what the pops after the first T leaves can take
+__host__ __device__ inline int prio_cap(int budget, int T) { return budget > T ? budget - T : 1; }
 
-// per-warp shared memory: the large queue array (`budget` + 64 entries), the small one (two
-// buffers), the staged batch and its sorted copy, then one reflection weight per tree
-__host__ __device__ inline size_t prio_warp_bytes(int budget, int T) {
-    return (size_t)(budget + 64 + 2 * PQ_BCAP + 64) * sizeof(PQE) + (size_t)(T + 3) / 4 * 16;
+// per-warp shared memory: the two arrays' keys, then their places, then one reflection weight per tree
+__host__ __device__ inline size_t prio_warp_bytes(int budget, int T, size_t place) {
+    const size_t n = prio_cap(budget, T) + PQ_BCAP;
+    return (n * 8 + n * place + (size_t)T * 4 + 15) / 16 * 16;
 }
 
+template <typename Place>
 __global__ void __launch_bounds__(PRIO_WARPS * 32) k_prio_leaves(ForestView F, const float *__restrict__ Q,
-                                                                long long m, int budget, int cap,
-                                                                unsigned *leaves, int *nleaves) {
+                                                                long long m, int budget, unsigned *leaves, int *nleaves) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned char *mine = smem_raw + (size_t)w * prio_warp_bytes(budget, F.T);
-    PQE *base = reinterpret_cast<PQE *>(mine);
-    PQE *qa = base;                                   // A [cap]
-    PQE *qb = base + cap, *qb2 = qb + PQ_BCAP;        // B, double-buffered
-    PQE *stage = qb2 + PQ_BCAP, *sorted = stage + 32;
-    float *w2s = reinterpret_cast<float *>(sorted + 32);
+    const int cap = prio_cap(budget, F.T);
+    PQArray<Place> qa, qb;
+    qa.key = reinterpret_cast<unsigned long long *>(smem_raw + (size_t)w * prio_warp_bytes(budget, F.T, sizeof(Place)));
+    qb.key = qa.key + cap;
+    qa.at = reinterpret_cast<Place *>(qb.key + PQ_BCAP);
+    qb.at = qa.at + cap;
+    float *w2s = reinterpret_cast<float *>(qb.at + PQ_BCAP);
     const int nn = (1 << F.L) - 1;
     const int nwq = blockDim.x >> 5;
     for (long long qi = (long long)blockIdx.x * nwq + w; qi < m; qi += (long long)gridDim.x * nwq) {
@@ -190,23 +213,20 @@ __global__ void __launch_bounds__(PRIO_WARPS * 32) k_prio_leaves(ForestView F, c
             }
             int j = 0;
             for (int l = 0; l < F.L; ++l) {
-                PQE e = pq_inf();
+                PQE<Place> e = pq_inf<Place>();
                 if (act) {
                     const int2 nd = __ldg(F.nodes + (size_t)t * F.nnodes + j);
                     const float qx = __ldg(q + nd.x);
                     const float qs = F.U ? reflect_coord(qx, w2, __ldg(F.U + (size_t)t * F.d + nd.x)) : qx;
                     const float v = __int_as_float(nd.y);
+                    const bool left = qs < v;
                     e.key = pq_key(qs, v);
-                    e.tree = t;
-                    e.node = qs < v ? 2 * j + 2 : 2 * j + 1;  // the child not taken
-                    j = qs < v ? 2 * j + 1 : 2 * j + 2;
+                    e.at = ((Place)t << (F.L + 1)) | (Place)(left ? 2 * j + 2 : 2 * j + 1);  // the child not taken
+                    j = left ? 2 * j + 1 : 2 * j + 2;
                 }
-                stage[lane] = e;
-                __syncwarp();
                 const int nb = min(32, F.T - t0);
-                const int keep = min(cap, max(0, budget - F.T));
-                pq_sort_stage(stage, nb, sorted);
-                acnt = pq_merge_into(qa, acnt, sorted, nb, keep);
+                pq_insert(qb, 0, 0, e, nb, PQ_BCAP);
+                acnt = pq_merge_into(qa, acnt, qb, nb, max(0, budget - F.T));
             }
             if (act && t < budget) out[t] = leaf_code(t, j - nn, F.L);
         }
@@ -214,21 +234,22 @@ __global__ void __launch_bounds__(PRIO_WARPS * 32) k_prio_leaves(ForestView F, c
         // ---- pops in queue order
         while (checked < budget && (ahead < acnt || bhead < bcnt)) {
             // the smaller head of A and B
-            const PQE ta = ahead < acnt ? qa[ahead] : pq_inf(), tb = bhead < bcnt ? qb[bhead] : pq_inf();
+            const PQE<Place> ta = ahead < acnt ? qa.get(ahead) : pq_inf<Place>(), tb = bhead < bcnt ? qb.get(bhead) : pq_inf<Place>();
             const bool fromb = pq_less(tb, ta);
-            const PQE top = fromb ? tb : ta;
+            const Place top = fromb ? tb.at : ta.at;
             if (fromb) ++bhead;
             else ++ahead;
-            // descend from the popped node, staging the siblings passed.  The warp loads the
+            // descend from the popped node, lane i keeping the i-th sibling passed.  The warp loads the
             // five-level subtree below the current node at once (lane i: node i in breadth-first
             // order, with its query coordinate), then walks it through shuffles: five levels cost
             // one round of loads instead of five dependent ones.  Same path, same pushes.
-            const int tr = top.tree;
+            const int tr = (int)(top >> (F.L + 1));
             const int2 *tnodes = F.nodes + (size_t)tr * F.nnodes;
             const float *u = F.U ? F.U + (size_t)tr * F.d : nullptr;
             const float w2 = u ? w2s[tr] : 0.f;
             const int lv = 31 - __clz(lane + 1);  // lane's level in the subtree (lanes 0..30)
-            int j = top.node, nb = 0;
+            int j = (int)(top & (((Place)2 << F.L) - 1)), nb = 0;
+            PQE<Place> mine = pq_inf<Place>();
             while (j < nn) {
                 const long long node = (((long long)j + 1) << lv) - 1 + (lane + 1 - (1 << lv));
                 float qs_l = 0.f, v_l = 0.f;
@@ -238,17 +259,15 @@ __global__ void __launch_bounds__(PRIO_WARPS * 32) k_prio_leaves(ForestView F, c
                     qs_l = u ? reflect_coord(qx, w2, __ldg(u + nd.x)) : qx;
                     v_l = __int_as_float(nd.y);
                 }
+                const unsigned lefts = __ballot_sync(FULL, qs_l < v_l);
+                const unsigned long long key_l = pq_key(qs_l, v_l);  // of every node, before the walk picks
                 int bi = 0;  // breadth-first index of the current node in the loaded subtree
                 for (int l = 0; l < 5 && j < nn; ++l) {
-                    const float qs = __shfl_sync(FULL, qs_l, bi);
-                    const float v = __shfl_sync(FULL, v_l, bi);
-                    const bool left = qs < v;
-                    if (lane == 0) {
-                        PQE e;
-                        e.key = pq_key(qs, v);
-                        e.tree = tr;
-                        e.node = left ? 2 * j + 2 : 2 * j + 1;
-                        stage[nb] = e;
+                    const unsigned long long key = __shfl_sync(FULL, key_l, bi);
+                    const bool left = (lefts >> bi) & 1u;
+                    if (lane == nb) {
+                        mine.key = key;
+                        mine.at = ((Place)tr << (F.L + 1)) | (Place)(left ? 2 * j + 2 : 2 * j + 1);
                     }
                     ++nb;
                     j = left ? 2 * j + 1 : 2 * j + 2;
@@ -256,16 +275,13 @@ __global__ void __launch_bounds__(PRIO_WARPS * 32) k_prio_leaves(ForestView F, c
                 }
             }
             if (lane == 0) out[checked] = leaf_code(tr, j - nn, F.L);
-            __syncwarp();
             ++checked;
             // the pushes go to B (its popped prefix dropped); keep only what later pops can take
             const int keep = max(0, budget - checked);
-            bcnt = pq_merge(qb + bhead, bcnt - bhead, stage, nb, qb2, min(PQ_BCAP, keep), sorted);
+            bcnt = pq_insert(qb, bhead, bcnt - bhead, mine, nb, min(PQ_BCAP, keep));
             bhead = 0;
-            PQE *tmp = qb; qb = qb2; qb2 = tmp;
-            __syncwarp();
             if (bcnt > PQ_BCAP - 32) {  // the next pushes might not fit: B into A
-                acnt = ahead + pq_merge_into(qa + ahead, acnt - ahead, qb, bcnt, keep);
+                acnt = ahead + pq_merge_into(qa.from(ahead), acnt - ahead, qb, bcnt, keep);
                 bcnt = 0;
             }
         }
@@ -274,25 +290,30 @@ __global__ void __launch_bounds__(PRIO_WARPS * 32) k_prio_leaves(ForestView F, c
     }
 }
 
-}  // namespace
-
-size_t gf_prio_smem_bytes(int budget, int T) { return prio_warp_bytes(budget, T); }
-
-int gf_launch_prio_leaves(const gf_forest *F, const float *Q, int64_t m, int budget, unsigned *leaves,
-                          int *nleaves, cudaStream_t st) {
-    const int cap = budget + 64;
+template <typename Place>
+int launch_prio(const gf_forest *F, const float *Q, int64_t m, int budget, unsigned *leaves, int *nleaves, cudaStream_t st) {
     int dev = 0, lim = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const size_t per_warp = prio_warp_bytes(budget, F->T);
+    const size_t per_warp = prio_warp_bytes(budget, F->T, sizeof(Place));
     const int warps = (int)std::min<size_t>(PRIO_WARPS, (size_t)lim / per_warp);
     if (warps < 1) return gf_fail(GF_EUNSUPPORTED, "leaf budget %d needs %zu B of shared memory", budget, per_warp);
     const size_t smem = per_warp * warps;
-    if (smem > 48 * 1024) GF_CUDA_TRY(cudaFuncSetAttribute(k_prio_leaves, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const long long blocks = std::min<long long>((m + warps - 1) / warps, (long long)F->num_sms * 16);
-    k_prio_leaves<<<(unsigned)blocks, warps * 32, smem, st>>>(view_of(F), Q, m, budget, cap, leaves, nleaves);
+    if (smem > 48 * 1024)
+        GF_CUDA_TRY(cudaFuncSetAttribute(k_prio_leaves<Place>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const long long blocks = std::min<long long>((m + warps - 1) / warps, (long long)F->num_sms * 256);
+    k_prio_leaves<Place><<<(unsigned)blocks, warps * 32, smem, st>>>(view_of(F), Q, m, budget, leaves, nleaves);
     GF_CUDA_TRY(cudaGetLastError());
     return GF_OK;
+}
+
+}  // namespace
+
+int gf_launch_prio_leaves(const gf_forest *F, const float *Q, int64_t m, int budget, unsigned *leaves,
+                          int *nleaves, cudaStream_t st) {
+    return ((unsigned long long)F->T << (F->L + 1)) <= (1ull << 32)
+               ? launch_prio<uint32_t>(F, Q, m, budget, leaves, nleaves, st)
+               : launch_prio<unsigned long long>(F, Q, m, budget, leaves, nleaves, st);
 }
 
 extern "C" int gf_prio_leaves(const gf_forest *F, const float *Q, int64_t m, int32_t checks, double eps,
