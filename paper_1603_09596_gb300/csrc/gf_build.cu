@@ -303,9 +303,11 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 
 // ---------------------------------------------------------------- variance bounds in fixed point
 //
-// Coordinate j of every point as q = rint((x - mid_j) / s_j), 16 bits, s_j = range_j / 65000.  Rounding
-// moves a coordinate by at most QERR s_j (half a step, plus the float32 rounding of x - mid_j and of
-// the product, under 0.01 of a step at |q| <= 32,500), so over a node of c points the square root of
+// Coordinate j of every point as q = rint((x - low_j) / s_j) - 32500, 16 bits, s_j = range_j / 65000.
+// (From the smallest value, not the middle: a dimension that spans few float32 steps has no middle to
+// that precision, and q would leave 16 bits.)  Rounding moves a coordinate by at most QERR s_j (half
+// a step, plus the float32 rounding of x - low_j, of the product and of 1 / s_j against s_j, together
+// under 0.02 of a step at 65,000 steps), so over a node of c points the square root of
 // the sum of squared deviations moves by at most QERR sqrt(c) s_j (triangle inequality), which bounds
 // the variance on both sides.  A level's sums read 2 bytes a coordinate instead of 4 and cost a few
 // integer instructions instead of some 26 of compensated float32: 500,000 x 960, T = 32, a level took
@@ -315,6 +317,7 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 constexpr int CAND_MAX = 64;       // dimensions listed per node; -1: more, the node is summed in full
 constexpr float QERR = 0.52f;
 constexpr float QSTEPS = 65000.f;  // s_j = range_j / QSTEPS
+constexpr int QBIAS = 32500;       // half of them
 constexpr int QCHUNK = 2048;       // points a CTA sums
 constexpr long long QSUM_BYTES = 1ll << 30;  // sums kept for a level's nodes (and its parents')
 
@@ -339,8 +342,8 @@ __global__ void __launch_bounds__(256) k_range(const float *__restrict__ x, long
     atomicMax(rng + d + j, range_bits(hi));
 }
 
-// qdim[j] = (mid, 1 / s, s); s = 0: a constant dimension; s < 0: a range outside [1e-30, 1e30], whose
-// variance is left unknown (q = 0)
+// qdim[j] = (low, 1 / s, s); s = 0: a constant dimension; s < 0: a range outside [1e-30, 1e30], whose
+// variance is left unknown (every q the same)
 __global__ void k_qdim(const unsigned *__restrict__ rng, int d, float4 *qdim) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= d) return;
@@ -348,7 +351,7 @@ __global__ void k_qdim(const unsigned *__restrict__ rng, int d, float4 *qdim) {
     const float range = hi - lo;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
     if (range != 0.f) {
-        if (range >= 1e-30f && range <= 1e30f) q = make_float4(lo + 0.5f * range, QSTEPS / range, range / QSTEPS, 0.f);
+        if (range >= 1e-30f && range <= 1e30f) q = make_float4(lo, QSTEPS / range, range / QSTEPS, 0.f);
         else q.z = -1.f;
     }
     qdim[j] = q;
@@ -368,7 +371,7 @@ __global__ void __launch_bounds__(256) k_quant(const float *__restrict__ x, long
             int q = 0;
             if (j < d) {
                 const float4 p = __ldg(qdim + j);
-                q = __float2int_rn((__ldg(x + i * ldx + j) - p.x) * p.y);
+                q = __float2int_rn((__ldg(x + i * ldx + j) - p.x) * p.y) - QBIAS;
             }
             if (u & 1) w[u / 2] |= (unsigned)q << 16;
             else w[u / 2] = (unsigned)q & 0xffffu;

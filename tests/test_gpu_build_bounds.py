@@ -60,3 +60,18 @@ def test_build_derived_sums_agree_with_direct_ones(gf):
     G, Fg = gpu_build(gf, X, 4, 2, seed=6)
     Fo = oracle.build_forest(X, 4, 2, seed=6)
     assert_same_forest(X, Fg, Fo, 5)
+
+
+@pytest.mark.parametrize("most", [1, 3, 90])  # float32 steps a dimension spans
+@pytest.mark.parametrize("n,d,T,p", [(20_011, 101, 3, 40), (9000, 1100, 2, 300)])
+def test_build_on_few_float32_steps_equals_the_shifted_build(gf, most, n, d, T, p):
+    """Small even integers on 2^24, where float32 steps by 2: all differences between points, and so
+    the sums, the choices and the order, are those of the integers themselves."""
+    rng = np.random.default_rng(n + most)
+    span = rng.integers(1, most + 1, d)
+    X = 2.0 * rng.binomial(span, rng.uniform(0.05, 0.95, d), (n, d))
+    _, A = gpu_build(gf, np.ascontiguousarray(X, dtype=np.float32), T, p, seed=5)
+    _, B = gpu_build(gf, np.ascontiguousarray(X + 2.0 ** 24, dtype=np.float32), T, p, seed=5)
+    assert np.array_equal(A.split_dim, B.split_dim)
+    assert np.array_equal(A.perm, B.perm)
+    assert np.array_equal(A.split_val + np.float32(2.0 ** 24), B.split_val)
