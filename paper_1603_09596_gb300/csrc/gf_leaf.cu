@@ -1149,8 +1149,17 @@ constexpr int MERGE_NT = 256;
 constexpr int MERGE_SLOTS = 2048;  // of the hash set
 constexpr int MERGE_IDS = 1024;    // ids it takes
 
-size_t merge_smem(const gf_forest *F, int rerank) {
-    return (size_t)MERGE_SLOTS * 12 + (size_t)MERGE_IDS * 8 + (rerank ? (size_t)ldq_of(F->d) * 4 : 0);
+constexpr int MERGE_SET_BYTES = MERGE_SLOTS * 12 + MERGE_IDS * 8;
+
+// A query row longer than the set comes in after the selection, over the set (all but its first
+// entries are done with): rows of up to 227 KB less a few bytes fit, as many as without a set.
+__host__ __device__ inline bool merge_late(int d) { return ldq_of(d) * 4 > MERGE_SET_BYTES; }
+__host__ __device__ inline int merge_late_at(int R) { return (R * 12 + 15) / 16 * 16; }
+
+size_t merge_smem(const gf_forest *F, int R, int rerank) {
+    const size_t row = (size_t)ldq_of(F->d) * 4;
+    if (!rerank) return MERGE_SET_BYTES;
+    return merge_late(F->d) ? std::max<size_t>(MERGE_SET_BYTES, merge_late_at(R) + row) : MERGE_SET_BYTES + row;
 }
 
 template <int NCF>
@@ -1160,11 +1169,12 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
                                                             const unsigned long long *__restrict__ tau, long long *ids,
                                                             float *dists) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned long long *hkey = reinterpret_cast<unsigned long long *>(smem_raw);  // [MERGE_SLOTS]
-    unsigned long long *a = hkey + MERGE_SLOTS;                                   // [MERGE_IDS]
-    int *hid = reinterpret_cast<int *>(a + MERGE_IDS);                            // [MERGE_SLOTS]
-    float *qs = reinterpret_cast<float *>(hid + MERGE_SLOTS);                     // [ldq], rerank only
-    __shared__ int sid[R_MAX];
+    unsigned long long *a = reinterpret_cast<unsigned long long *>(smem_raw);  // [MERGE_IDS]
+    unsigned long long *hkey = a + MERGE_IDS;                                  // [MERGE_SLOTS]
+    int *hid = reinterpret_cast<int *>(hkey + MERGE_SLOTS);                    // [MERGE_SLOTS]
+    int *sid = reinterpret_cast<int *>(a + R);                                 // [R], after the selection
+    const bool late = merge_late(F.d);
+    float *qs = reinterpret_cast<float *>(late ? smem_raw + merge_late_at(R) : smem_raw + MERGE_SET_BYTES);  // [ldq], rerank only
     __shared__ unsigned long long sbound;
     __shared__ int nheld, nids;
     const int TR = S * R, tid = threadIdx.x;
@@ -1187,7 +1197,7 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
             for (int u = 0; u < 8; ++u)
                 if (kv[u] < mn && usable(kv[u], tq)) mn = kv[u];
         }
-        if (rerank) load_query(Q + qi * F.d, F.d, qs);
+        if (rerank && !late) load_query(Q + qi * F.d, F.d, qs);
         // the smallest keys of different ids: drop a thread's if another thread has the id at a smaller key
         hkey[tid] = mn;
         if (tid == 0) sbound = tq;
@@ -1263,6 +1273,7 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
         const int C = min(R, n);
         if (rerank) {
             for (int i = tid; i < C; i += MERGE_NT) sid[i] = (int)(unsigned)(a[i] & 0xffffffffu);
+            if (late) load_query(Q + qi * F.d, F.d, qs);
             __syncthreads();
             rescore_f32<NCF>(F, qs, sid, C, a);
             sort_distinct(a, C);
@@ -1502,7 +1513,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "leaf-major scoring launch");
     if (events && (e = cudaEventRecord(events[1], st)) != cudaSuccess) return fail(e, "cudaEventRecord");
 
-    const size_t msmem = merge_smem(F, !f32);
+    const size_t msmem = merge_smem(F, R, !f32);
     const unsigned mg = (unsigned)std::min<long long>(m, (long long)F->num_sms * 64);
     const int ncf = F->ldx / 4 <= 32 ? 1 : F->ldx / 4 <= 64 ? 2 : F->ldx / 4 <= 128 ? 4 : F->ldx / 4 <= 256 ? 8 : 0;
 #define GF_MERGE(NCV)                                                                                    \

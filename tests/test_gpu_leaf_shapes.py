@@ -56,3 +56,21 @@ def test_leaf_screen_shapes(gf, leaf, leaves, d, m, prec, ctas):
     offs, ids = oracle.candidates(F, oracle.descend(F, Q))
     oi, od, _ = screen.screened_search(F, X, Q, 8, 24, prec, offs, ids)
     assert_screened_close(X, Q, gi.cpu().numpy(), gd.cpu().numpy(), oi, od, offs, ids, prec, 24, "norm")
+
+
+@pytest.mark.parametrize("d", [8177, 8208, 50_001, 56_000])
+@pytest.mark.parametrize("precision", ["bf16", "fp8"])
+def test_leaf_merge_rescores_long_rows(gf, d, precision):
+    """Rows on both sides of the merge's own set in length, up to what a CTA's shared memory holds.
+    One leaf of well separated points: the k nearest of all, which any screen keeps."""
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((60, d)).astype(np.float32)
+    Q = X[:12] + rng.standard_normal((12, d)).astype(np.float32) * np.float32(0.01)
+    G = gf.gf_build(torch.from_numpy(X).cuda(), 1, 64, t=1)
+    prec = {"bf16": gf.GF_BF16_RERANK, "fp8": gf.GF_FP8_RERANK}[precision]
+    gf.gf_forest_add_screen(G, prec)
+    ids, dists = gf.gf_query(G, torch.from_numpy(Q).cuda(), 1, precision=prec, rerank_R=32, algo=gf.GF_ALGO_LEAF)
+    want = np.square(X[:12].astype(np.float64) - Q).sum(1)
+    assert ids.cpu().numpy()[:, 0].tolist() == list(range(12))
+    # float32 sums of d squares by 32 lanes: at most d / 32 + 10 roundings of 2^-24 each
+    assert np.all(np.abs(dists.cpu().numpy()[:, 0] - want) <= want * (d / 32 + 10) * 2.0 ** -24)
