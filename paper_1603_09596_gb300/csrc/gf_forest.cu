@@ -197,6 +197,8 @@ int gf_forest_alloc(gf_forest **out, const float *X, int64_t n, int32_t d, int32
     if ((r = gf_dmalloc((void **)&F->nodes, (size_t)T * nn * sizeof(int2)))) { forest_release(F); return r; }
     if ((r = gf_dmalloc((void **)&F->perm, (size_t)T * n * 4))) { forest_release(F); return r; }
     F->device_bytes = (borrow ? 0 : (int64_t)n * F->ldx * 4) + (int64_t)(T * nn * sizeof(int2)) + (int64_t)T * n * 4;
+    cudaMemPool_t pool;  // made here, so that a query under stream capture does not
+    if (scratch_pool(&pool) != cudaSuccess) cudaGetLastError();
     {
         std::lock_guard<std::mutex> g(g_pool_mu);
         F->live = true;
