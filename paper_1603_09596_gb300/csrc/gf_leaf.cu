@@ -1138,43 +1138,54 @@ __global__ void k_qsplit8(const float *__restrict__ Q, long long m, int d, int l
 // nearest.  One CTA per query at a time.
 //
 // The lists hold S R keys (8192 at the most) at or below the bounds their chunks knew, the same id in
-// many of them; the R best ids are a few dozen keys and their copies.  The keys are dealt to the
-// threads, and the R-th smallest of the threads' smallest keys of different ids bounds the R-th best
-// id from above.  The keys at or below that go into a hash set by id that keeps each id's smallest
-// key.  Should more than MERGE_IDS ids lie below the bound, the R-th smallest key held (of as many
-// different ids) is a lower one, and the keys are gathered again.  The lists are read twice (the second
-// time from L2) and nothing is sorted but the few keys left: 10^4 queries of 8192 keys took 5.26 ms
-// with all keys below tau_q sorted twice in shared memory (1024 keys each and R = 32: 0.82 ms).
-constexpr int MERGE_NT = 256;
-constexpr int MERGE_SLOTS = 2048;  // of the hash set
-constexpr int MERGE_IDS = 1024;    // ids it takes
+// many of them; the R best ids are a few dozen keys and their copies.  The keys at or below a bound
+// go into a hash set by id that keeps each id's smallest key, and the ids held are sorted.
+// SMALL (S R <= MERGE_SMALL): the bound is tau_q and the set holds all keys that there can be; 128 threads.
+// Else the keys are dealt to 256 threads, and the R-th smallest of the threads' smallest keys of
+// different ids bounds the R-th best id from above.  Should more than MERGE_IDS ids lie below the
+// bound, the R-th smallest key held (of as many different ids) is a lower one, and the keys are
+// gathered again.  The lists are read twice then (the second time from L2).
+// Microseconds a search of 10^4 queries, two sorts of all keys below tau_q in shared memory / 256 threads
+// and a bound at every size / now: T = 8, R = 16 (50,000 x 300) 656 / 992 / 535; T = 32, R = 24 (100,000 x 300)
+// 2465 / 2474 / 2125; T = 32, R = 32 (300,000 x 960) 5241 / 4889 / 4594.  8192 keys (512 leaves, R = 16):
+// the merge alone 5260 / 710.
+constexpr int MERGE_SMALL = 1024;  // keys
+constexpr int MERGE_SLOTS = 2048;  // of the hash set; SMALL: the power of two of at least twice the keys
+constexpr int MERGE_IDS = 1024;    // ids it takes; SMALL: half the slots
 
-constexpr int MERGE_SET_BYTES = MERGE_SLOTS * 12 + MERGE_IDS * 8;
-
-// A query row longer than the set comes in after the selection, over the set (all but its first
-// entries are done with): rows of up to 227 KB less a few bytes fit, as many as without a set.
-__host__ __device__ inline bool merge_late(int d) { return ldq_of(d) * 4 > MERGE_SET_BYTES; }
-__host__ __device__ inline int merge_late_at(int R) { return (R * 12 + 15) / 16 * 16; }
-
-size_t merge_smem(const gf_forest *F, int R, int rerank) {
-    const size_t row = (size_t)ldq_of(F->d) * 4;
-    if (!rerank) return MERGE_SET_BYTES;
-    return merge_late(F->d) ? std::max<size_t>(MERGE_SET_BYTES, merge_late_at(R) + row) : MERGE_SET_BYTES + row;
+int merge_slots(int TR) {
+    int slots = 64;
+    while (slots < MERGE_SLOTS && slots < 2 * TR) slots <<= 1;
+    return TR <= MERGE_SMALL ? slots : MERGE_SLOTS;
 }
 
-template <int NCF>
-__global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const float *__restrict__ Q, long long m, int k,
-                                                            int R, int S, int rerank,
-                                                            const unsigned long long *__restrict__ part,
-                                                            const unsigned long long *__restrict__ tau, long long *ids,
-                                                            float *dists) {
+// A query row longer than the largest set comes in after the selection, over the set (all but its first
+// entries are done with): rows of up to 227 KB less a few bytes fit, as many as without a set.
+__host__ __device__ inline bool merge_late(int d) { return ldq_of(d) * 4 > MERGE_SLOTS * 16; }
+__host__ __device__ inline int merge_late_at(int R) { return (R * 12 + 15) / 16 * 16; }
+
+size_t merge_smem(const gf_forest *F, int R, int slots, int rerank) {
+    const size_t row = (size_t)ldq_of(F->d) * 4, set = (size_t)slots * 16;
+    if (!rerank) return set;
+    return merge_late(F->d) ? std::max<size_t>(set, merge_late_at(R) + row) : set + row;
+}
+
+template <int NCF, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 128 : 256, SMALL ? 6 : 3)
+    k_leaf_merge(ForestView F, const float *__restrict__ Q, long long m, int k, int R, int S, int rerank, int nslots,
+                 const unsigned long long *__restrict__ part, const unsigned long long *__restrict__ tau, long long *ids,
+                 float *dists) {
+    constexpr int NT = SMALL ? 128 : 256;
+    constexpr int U = SMALL ? MERGE_SMALL / NT : 8;  // keys a thread has in flight
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned long long *a = reinterpret_cast<unsigned long long *>(smem_raw);  // [MERGE_IDS]
-    unsigned long long *hkey = a + MERGE_IDS;                                  // [MERGE_SLOTS]
-    int *hid = reinterpret_cast<int *>(hkey + MERGE_SLOTS);                    // [MERGE_SLOTS]
+    const int slots = SMALL ? nslots : MERGE_SLOTS, most = SMALL ? nslots / 2 : MERGE_IDS;
+    const int shift = 32 - (31 - __clz(slots));  // the hash's top log2(slots) bits
+    unsigned long long *a = reinterpret_cast<unsigned long long *>(smem_raw);  // [most]
+    unsigned long long *hkey = a + most;                                       // [slots]
+    int *hid = reinterpret_cast<int *>(hkey + slots);                          // [slots]
     int *sid = reinterpret_cast<int *>(a + R);                                 // [R], after the selection
     const bool late = merge_late(F.d);
-    float *qs = reinterpret_cast<float *>(late ? smem_raw + merge_late_at(R) : smem_raw + MERGE_SET_BYTES);  // [ldq], rerank only
+    float *qs = reinterpret_cast<float *>(smem_raw + (late ? merge_late_at(R) : slots * 16));  // [ldq], rerank only
     __shared__ unsigned long long sbound;
     __shared__ int nheld, nids;
     const int TR = S * R, tid = threadIdx.x;
@@ -1185,37 +1196,45 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
         auto usable = [&](unsigned long long key, unsigned long long bound) {
             return key != KEY_NONE && key <= bound && (key & 0xffffffffull) < (unsigned long long)F.n;
         };
-        unsigned long long mn = KEY_NONE;
-        for (int base = 0; base < TR; base += MERGE_NT * 8) {
-            unsigned long long kv[8];
+        unsigned long long kv[U];
+        auto read = [&](int base) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = base + u * MERGE_NT + tid;
+            for (int u = 0; u < U; ++u) {
+                const int i = base + u * NT + tid;
                 kv[u] = i < TR ? __ldcg(pq + i) : KEY_NONE;
             }
+        };
+        if (SMALL) {
+            read(0);  // all of them
+            if (rerank && !late) load_query(Q + qi * F.d, F.d, qs);
+        } else {
+            unsigned long long mn = KEY_NONE;
+            for (int base = 0; base < TR; base += NT * U) {
+                read(base);
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (kv[u] < mn && usable(kv[u], tq)) mn = kv[u];
+                for (int u = 0; u < U; ++u)
+                    if (kv[u] < mn && usable(kv[u], tq)) mn = kv[u];
+            }
+            if (rerank && !late) load_query(Q + qi * F.d, F.d, qs);
+            // the smallest keys of different ids: drop a thread's if another thread has the id at a smaller key
+            hkey[tid] = mn;
+            if (tid == 0) sbound = tq;
+            __syncthreads();
+            bool copy = mn == KEY_NONE;
+            for (int j = 0; j < NT; ++j) {
+                const unsigned long long o = hkey[j];
+                copy |= (unsigned)o == (unsigned)mn && (o < mn || (o == mn && j < tid));
+            }
+            a[tid] = copy ? KEY_NONE : mn;
+            __syncthreads();
+            int rank = 0;
+            for (int j = 0; j < NT; ++j) rank += a[j] < mn;
+            if (!copy && rank == R - 1) sbound = mn;
+            __syncthreads();
         }
-        if (rerank && !late) load_query(Q + qi * F.d, F.d, qs);
-        // the smallest keys of different ids: drop a thread's if another thread has the id at a smaller key
-        hkey[tid] = mn;
-        if (tid == 0) sbound = tq;
-        __syncthreads();
-        bool copy = mn == KEY_NONE;
-        for (int j = 0; j < MERGE_NT; ++j) {
-            const unsigned long long o = hkey[j];
-            copy |= (unsigned)o == (unsigned)mn && (o < mn || (o == mn && j < tid));
-        }
-        a[tid] = copy ? KEY_NONE : mn;
-        __syncthreads();
-        int rank = 0;
-        for (int j = 0; j < MERGE_NT; ++j) rank += a[j] < mn;
-        if (!copy && rank == R - 1) sbound = mn;
-        __syncthreads();
         int n = 0;
-        for (unsigned long long bound = sbound;;) {
-            for (int i = tid; i < MERGE_SLOTS; i += MERGE_NT) {
+        for (unsigned long long bound = SMALL ? tq : sbound;;) {
+            for (int i = tid; i < slots; i += NT) {
                 hid[i] = -1;
                 hkey[i] = KEY_NONE;
             }
@@ -1224,26 +1243,21 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
                 nids = 0;
             }
             __syncthreads();
-            for (int base = 0; base < TR; base += MERGE_NT * 8) {
-                unsigned long long kv[8];
+            for (int base = 0; base < TR; base += NT * U) {
+                if (!SMALL) read(base);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = base + u * MERGE_NT + tid;
-                    kv[u] = i < TR ? __ldcg(pq + i) : KEY_NONE;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                for (int u = 0; u < U; ++u) {
                     if (!usable(kv[u], bound)) continue;
                     const int id = (int)(unsigned)kv[u];
-                    unsigned h = ((unsigned)id * 2654435769u) >> 21;  // the top 11 bits: MERGE_SLOTS slots
-                    // at most MERGE_IDS + MERGE_NT slots are ever taken, so the probe ends
+                    unsigned h = ((unsigned)id * 2654435769u) >> shift;
+                    // at most MERGE_IDS + NT slots (SMALL: half of them) are ever taken, so the probe ends
                     for (;;) {
                         int at = *reinterpret_cast<volatile int *>(hid + h);
                         if (at == -1) {
-                            if (*reinterpret_cast<volatile int *>(&nids) > MERGE_IDS) break;  // full: a lower bound comes
+                            if (!SMALL && *reinterpret_cast<volatile int *>(&nids) > MERGE_IDS) break;  // full: a lower bound comes
                             at = atomicCAS(hid + h, -1, id);
                             if (at == -1) {
-                                atomicAdd(&nids, 1);
+                                if (!SMALL) atomicAdd(&nids, 1);
                                 at = id;
                             }
                         }
@@ -1251,20 +1265,20 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
                             atomicMin(hkey + h, kv[u]);
                             break;
                         }
-                        h = (h + 1) & (MERGE_SLOTS - 1);
+                        h = (h + 1) & (slots - 1);
                     }
                 }
             }
             __syncthreads();
-            const bool full = nids > MERGE_IDS;
-            for (int i = tid; i < MERGE_SLOTS; i += MERGE_NT) {
+            const bool full = !SMALL && nids > MERGE_IDS;
+            for (int i = tid; i < slots; i += NT) {
                 if (hid[i] >= 0) {
                     const int at = atomicAdd(&nheld, 1);
-                    if (at < MERGE_IDS) a[at] = hkey[i];
+                    if (at < most) a[at] = hkey[i];
                 }
             }
             __syncthreads();
-            n = min(nheld, MERGE_IDS);
+            n = min(nheld, most);
             sort_distinct(a, n);
             if (!full) break;
             bound = a[R - 1];
@@ -1272,7 +1286,7 @@ __global__ void __launch_bounds__(MERGE_NT, 3) k_leaf_merge(ForestView F, const 
         }
         const int C = min(R, n);
         if (rerank) {
-            for (int i = tid; i < C; i += MERGE_NT) sid[i] = (int)(unsigned)(a[i] & 0xffffffffu);
+            for (int i = tid; i < C; i += NT) sid[i] = (int)(unsigned)(a[i] & 0xffffffffu);
             if (late) load_query(Q + qi * F.d, F.d, qs);
             __syncthreads();
             rescore_f32<NCF>(F, qs, sid, C, a);
@@ -1513,16 +1527,18 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "leaf-major scoring launch");
     if (events && (e = cudaEventRecord(events[1], st)) != cudaSuccess) return fail(e, "cudaEventRecord");
 
-    const size_t msmem = merge_smem(F, R, !f32);
+    const bool small = S * R <= MERGE_SMALL;
+    const int slots = merge_slots(S * R);
+    const size_t msmem = merge_smem(F, R, slots, !f32);
     const unsigned mg = (unsigned)std::min<long long>(m, (long long)F->num_sms * 64);
     const int ncf = F->ldx / 4 <= 32 ? 1 : F->ldx / 4 <= 64 ? 2 : F->ldx / 4 <= 128 ? 4 : F->ldx / 4 <= 256 ? 8 : 0;
 #define GF_MERGE(NCV)                                                                                    \
     if (ncf == NCV) {                                                                                    \
+        auto kern = small ? k_leaf_merge<NCV, true> : k_leaf_merge<NCV, false>;                          \
         if (msmem > 46 * 1024 &&                                                                         \
-            (e = cudaFuncSetAttribute(k_leaf_merge<NCV>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
-                                      (int)msmem)) != cudaSuccess)                                       \
+            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem)) != cudaSuccess) \
             return fail(e, "cudaFuncSetAttribute(k_leaf_merge)");                                        \
-        k_leaf_merge<NCV><<<mg, MERGE_NT, msmem, st>>>(view_of(F), Q, m, k, R, S, !f32, part, tau, (long long *)ids, dists); \
+        kern<<<mg, small ? 128 : 256, msmem, st>>>(view_of(F), Q, m, k, R, S, !f32, slots, part, tau, (long long *)ids, dists); \
     }
     GF_MERGE(1) GF_MERGE(2) GF_MERGE(4) GF_MERGE(8) GF_MERGE(0)
 #undef GF_MERGE
