@@ -357,22 +357,33 @@ __global__ void k_qdim(const unsigned *__restrict__ rng, int d, float4 *qdim) {
     qdim[j] = q;
 }
 
-// xq[i][j], rows padded with zeros to ldq = round_up(d, 8); a thread makes eight values
-__global__ void __launch_bounds__(256) k_quant(const float *__restrict__ x, long long n, int d, int ldx, int ldq,
+// xq[i][j], rows padded with zeros to ldq = round_up(d, 8).  tpr threads cover a row (or, blockIdx.y,
+// a part of it), eight values each, and walk down the rows, so a dimension's (low, 1 / s) stays in
+// registers and a warp reads and writes whole lines: bound by the bytes in and out (500,000 x 960:
+// 1.98 ms with every thread fetching the eight dimensions' constants anew).
+__global__ void __launch_bounds__(256) k_quant(const float *__restrict__ x, long long n, int d, int ldx, int ldq, int tpr,
                                                const float4 *__restrict__ qdim, short *xq) {
-    const long long total = n * (ldq / 8);
-    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
-        const long long i = g / (ldq / 8);
-        const int j0 = (int)(g - i * (ldq / 8)) * 8;
+    const int col = threadIdx.x & (tpr - 1), grp = threadIdx.x / tpr, ngrp = 256 / tpr;
+    const int j0 = (blockIdx.y * tpr + col) * 8;
+    if (j0 >= ldq) return;
+    float low[8], inv[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const float4 p = j0 + u < d ? __ldg(qdim + j0 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+        low[u] = p.x;
+        inv[u] = p.y;
+    }
+    const bool second = j0 + 4 < ldx;  // (ldx is a multiple of four, above j0)
+    const long long step = (long long)gridDim.x * ngrp;
+#pragma unroll 4
+    for (long long i = (long long)blockIdx.x * ngrp + grp; i < n; i += step) {
+        const float4 *src = reinterpret_cast<const float4 *>(x + i * ldx + j0);
+        const float4 a = __ldg(src), b = second ? __ldg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         unsigned w[4];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int j = j0 + u;
-            int q = 0;
-            if (j < d) {
-                const float4 p = __ldg(qdim + j);
-                q = __float2int_rn((__ldg(x + i * ldx + j) - p.x) * p.y) - QBIAS;
-            }
+            const int q = j0 + u < d ? __float2int_rn((v[u] - low[u]) * inv[u]) - QBIAS : 0;
             if (u & 1) w[u / 2] |= (unsigned)q << 16;
             else w[u / 2] = (unsigned)q & 0xffffu;
         }
@@ -1055,7 +1066,9 @@ cudaError_t quant_prepare(QuantScratch &S, const BuildParams &P, long long wides
     const int rows = 256;
     k_range<<<dim3((unsigned)((P.n + rows - 1) / rows), (d + 255) / 256), 256, 0, st>>>(P.x, P.n, d, P.ldx, rows, (unsigned *)S.rng.p);
     k_qdim<<<(d + 255) / 256, 256, 0, st>>>((const unsigned *)S.rng.p, d, (float4 *)S.qdim.p);
-    k_quant<<<sms * 16, 256, 0, st>>>(P.x, P.n, d, P.ldx, S.ldq, (const float4 *)S.qdim.p, (short *)S.xq.p);
+    const int dblocks = (S.ldq + S.tpr * 8 - 1) / (S.tpr * 8);
+    k_quant<<<dim3((unsigned)(sms * 8), dblocks), 256, 0, st>>>(P.x, P.n, d, P.ldx, S.ldq, S.tpr, (const float4 *)S.qdim.p,
+                                                              (short *)S.xq.p);
     return cudaGetLastError();
 }
 

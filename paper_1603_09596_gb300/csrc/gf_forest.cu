@@ -355,69 +355,131 @@ extern "C" int gf_forest_set_tuning(gf_forest *F, int32_t precision, int32_t war
 
 // ---------------------------------------------------------------- screening copies
 
-// xb[i][j] = bf16_rne(x[i][j]) for j < d, 0 in the padding.
-__global__ void k_to_bf16(const float *__restrict__ x, int ldx, long long n, int d, int ldb,
-                          __nv_bfloat16 *xb) {
-    const long long total = n * ldb;
-    for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-         g += (long long)gridDim.x * blockDim.x) {
-        const long long i = g / ldb;
-        const int j = (int)(g - i * ldb);
-        xb[g] = __float2bfloat16_rn(j < d ? x[i * ldx + j] : 0.f);
+// A lane's share of a row's squared norm: float32 squares (exact in range: at most 16 significant bits)
+// summed as a float32 pair and added to a float64 sum at least every 32 squares.  The float64 conversion and
+// multiply-add of every value took most of the copies' time (GB300's float64 rate).
+struct SquareSum {
+    float hi = 0.f, lo = 0.f;
+    double acc = 0.0;
+    __device__ __forceinline__ void add(float v) {
+        const float p = __fmul_rn(v, v), s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ void flush() {
+        acc += hi;
+        acc += lo;
+        hi = lo = 0.f;
+    }
+    __device__ __forceinline__ double warp_total() {
+        flush();
+        double a = acc;
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        return a;
+    }
+};
+
+// Four values of a row from column j on, zeros past d (rows are 16-byte aligned, ldx a multiple of four).
+__device__ __forceinline__ float4 row4(const float *r, int j, int d, int ldx) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j < ldx) v = __ldg(reinterpret_cast<const float4 *>(r + j));
+    if (j + 1 > d) v.x = 0.f;
+    if (j + 2 > d) v.y = 0.f;
+    if (j + 3 > d) v.z = 0.f;
+    if (j + 4 > d) v.w = 0.f;
+    return v;
+}
+
+// xb[i][j] = bf16_rne(x[i][j]) for j < d, 0 in the padding; xbn[i] = sum_j xb[i][j]^2, rounded once.  A warp
+// per row, eight values a lane at a time, up to eight 16-byte loads in flight: bound by the row's
+// bytes in and out (500,000 x 960: 3.09 ms as two passes of scalar loads).
+__global__ void __launch_bounds__(256) k_to_bf16(const float *__restrict__ x, int ldx, long long n, int d, int ldb,
+                                                 __nv_bfloat16 *xb, float *xbn) {
+    const int lane = threadIdx.x & 31;
+    for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
+         i += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const float *r = x + i * ldx;
+        SquareSum sum;
+        for (int j0 = 0; j0 < ldb; j0 += 1024) {
+            float4 v[4][2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + 256 * u + 8 * lane;
+                v[u][0] = row4(r, j, d, ldx);
+                v[u][1] = row4(r, j + 4, d, ldx);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + 256 * u + 8 * lane;
+                __nv_bfloat162 b[4] = {__floats2bfloat162_rn(v[u][0].x, v[u][0].y), __floats2bfloat162_rn(v[u][0].z, v[u][0].w),
+                                       __floats2bfloat162_rn(v[u][1].x, v[u][1].y), __floats2bfloat162_rn(v[u][1].z, v[u][1].w)};
+                if (j < ldb) *reinterpret_cast<uint4 *>(xb + i * ldb + j) = *reinterpret_cast<const uint4 *>(b);
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const float2 f = __bfloat1622float2(b[h]);
+                    sum.add(f.x);
+                    sum.add(f.y);
+                }
+            }
+            sum.flush();
+        }
+        double total = sum.warp_total();
+        if (!(total > 1e-30 && total < 1e37)) {  // squares outside float32's range: every value in float64 (uniform)
+            total = 0.0;
+            for (int j = lane; j < d; j += 32) {
+                const double v = (double)__bfloat162float(__float2bfloat16_rn(__ldg(r + j)));
+                total += v * v;
+            }
+            for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        }
+        if (lane == 0) xbn[i] = (float)total;
     }
 }
 
-// One warp per row: a = max |x|, scale = a / 448, codes = e4m3_rne_satfinite(x * (448 / a)).
-__global__ void k_to_fp8(const float *__restrict__ x, int ldx, long long n, int d, int ld8, uint8_t *x8,
-                         float *scale) {
+// a = max |x|, scale = a / 448, codes = e4m3_rne_satfinite(x * (448 / a)), x8n[i] = sum_j (scale_i
+// x8[i][j])^2, rounded once.  A warp per row, sixteen values a lane at a time; the row is read again
+// for its codes, from the caches.
+__global__ void __launch_bounds__(256) k_to_fp8(const float *__restrict__ x, int ldx, long long n, int d, int ld8, uint8_t *x8,
+                                                float *scale, float *x8n) {
     const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long i = warp; i < n; i += nw) {
+    for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
+         i += ((long long)gridDim.x * blockDim.x) >> 5) {
         const float *r = x + i * ldx;
         float a = 0.f;
-        for (int j = lane; j < d; j += 32) a = fmaxf(a, fabsf(r[j]));
+#pragma unroll 8
+        for (int j = 4 * lane; j < d; j += 128) {
+            const float4 v = row4(r, j, d, ldx);
+            a = fmaxf(fmaxf(a, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
         const float inv = a > 0.f ? 448.0f / a : 0.f;
-        if (lane == 0) scale[i] = a > 0.f ? a / 448.0f : 1.0f;
-        for (int j = lane; j < ld8; j += 32) {
-            const float v = j < d ? r[j] * inv : 0.f;
-            x8[i * ld8 + j] = (uint8_t)__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3);
+        const float s = a > 0.f ? a / 448.0f : 1.0f;
+        if (lane == 0) scale[i] = s;
+        SquareSum sum;
+#pragma unroll 2
+        for (int j = 16 * lane; j < ld8; j += 512) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = row4(r, j + 4 * u, d, ldx);
+            unsigned w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float f[4] = {v[u].x * inv, v[u].y * inv, v[u].z * inv, v[u].w * inv};
+                w[u] = 0;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const __nv_fp8_storage_t c = __nv_cvt_float_to_fp8(f[h], __NV_SATFINITE, __NV_E4M3);
+                    w[u] |= (unsigned)c << (8 * h);
+                    const __half_raw hr = __nv_cvt_fp8_to_halfraw(c, __NV_E4M3);
+                    sum.add(__half2float(*reinterpret_cast<const __half *>(&hr)));
+                }
+            }
+            *reinterpret_cast<uint4 *>(x8 + i * ld8 + j) = make_uint4(w[0], w[1], w[2], w[3]);
+            sum.flush();
         }
-    }
-}
-
-// xbn[i] = sum_j xb[i][j]^2, accumulated in float64 and rounded once: a warp per row.
-__global__ void k_bf16_sqnorm(const __nv_bfloat16 *__restrict__ xb, long long n, int ldb, float *xbn) {
-    const int lane = threadIdx.x & 31;
-    for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
-         i += ((long long)gridDim.x * blockDim.x) >> 5) {
-        double acc = 0.0;
-        for (int j = lane; j < ldb; j += 32) {
-            const double v = (double)__bfloat162float(xb[i * ldb + j]);
-            acc += v * v;
-        }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) xbn[i] = (float)acc;
-    }
-}
-
-// x8n[i] = sum_j (scale_i x8[i][j])^2, accumulated in float64 and rounded once: a warp per row.
-__global__ void k_fp8_sqnorm(const uint8_t *__restrict__ x8, const float *__restrict__ scale, long long n, int ld8,
-                             float *x8n) {
-    const int lane = threadIdx.x & 31;
-    for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
-         i += ((long long)gridDim.x * blockDim.x) >> 5) {
-        double acc = 0.0;
-        for (int j = lane; j < ld8; j += 32) {
-            const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)x8[i * ld8 + j], __NV_E4M3);
-            const double v = (double)__half2float(*reinterpret_cast<const __half *>(&h));
-            acc += v * v;
-        }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        const double sc = (double)scale[i];
-        if (lane == 0) x8n[i] = (float)(acc * sc * sc);
+        const double total = sum.warp_total(), sc = (double)s;
+        if (lane == 0) x8n[i] = (float)(total * sc * sc);
     }
 }
 
@@ -430,8 +492,7 @@ extern "C" int gf_forest_add_screen(gf_forest *F, int32_t precision, void *strea
         if (F->xb) return GF_OK;
         if ((r = gf_dmalloc((void **)&F->xb, (size_t)F->n * F->ldb * 2))) return r;
         if ((r = gf_dmalloc((void **)&F->xbn, (size_t)F->n * 4))) { cudaFree(F->xb); F->xb = nullptr; return r; }
-        k_to_bf16<<<F->num_sms * 8, 256, 0, st>>>(F->x, F->ldx, F->n, F->d, F->ldb, F->xb);
-        k_bf16_sqnorm<<<F->num_sms * 8, 256, 0, st>>>(F->xb, F->n, F->ldb, F->xbn);
+        k_to_bf16<<<F->num_sms * 8, 256, 0, st>>>(F->x, F->ldx, F->n, F->d, F->ldb, F->xb, F->xbn);
         F->device_bytes += (int64_t)F->n * F->ldb * 2 + F->n * 4;
     } else if (precision == GF_FP8_RERANK) {
         if (F->x8) return GF_OK;
@@ -444,8 +505,7 @@ extern "C" int gf_forest_add_screen(gf_forest *F, int32_t precision, void *strea
             F->scale8 = nullptr;
             return r;
         }
-        k_to_fp8<<<F->num_sms * 8, 256, 0, st>>>(F->x, F->ldx, F->n, F->d, F->ld8, F->x8, F->scale8);
-        k_fp8_sqnorm<<<F->num_sms * 8, 256, 0, st>>>(F->x8, F->scale8, F->n, F->ld8, F->x8n);
+        k_to_fp8<<<F->num_sms * 8, 256, 0, st>>>(F->x, F->ldx, F->n, F->d, F->ld8, F->x8, F->scale8, F->x8n);
         F->device_bytes += (int64_t)F->n * F->ld8 + F->n * 8;
     } else {
         return gf_fail(GF_EINVAL, "precision %d has no screening copy", precision);

@@ -74,3 +74,20 @@ def test_leaf_merge_rescores_long_rows(gf, d, precision):
     assert ids.cpu().numpy()[:, 0].tolist() == list(range(12))
     # float32 sums of d squares by 32 lanes: at most d / 32 + 10 roundings of 2^-24 each
     assert np.all(np.abs(dists.cpu().numpy()[:, 0] - want) <= want * (d / 32 + 10) * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("scale", [1e-17, 1.0, 4e17])
+@pytest.mark.parametrize("d", [7, 300, 1025])
+def test_bf16_norms_of_small_and_large_values(gf, scale, d):
+    """The screen ranks by |x|^2 - 2 x q: norms whose squares leave float32's comfortable range."""
+    rng = np.random.default_rng(d)
+    s = np.float32(scale * (300 / d) ** 0.5)
+    X = rng.standard_normal((60, d)).astype(np.float32) * s
+    Q = X[:12] + rng.standard_normal((12, d)).astype(np.float32) * (s * np.float32(0.03))
+    G = gf.gf_build(torch.from_numpy(X).cuda(), 1, 64, t=1)
+    gf.gf_forest_add_screen(G, gf.GF_BF16_RERANK)
+    ids, dists = gf.gf_query(G, torch.from_numpy(Q).cuda(), 1, precision=gf.GF_BF16_RERANK, rerank_R=32, algo=gf.GF_ALGO_LEAF)
+    want = np.square(X[:12].astype(np.float64) - Q).sum(1)
+    assert ids.cpu().numpy()[:, 0].tolist() == list(range(12))
+    # float32 sums of d squares by 32 lanes, plus a float32 subnormal step a square
+    assert np.all(np.abs(dists.cpu().numpy()[:, 0] - want) <= want * (d / 32 + 10) * 2.0 ** -24 + d * 2.0 ** -148)
