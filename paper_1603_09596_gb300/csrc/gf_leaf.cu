@@ -1394,9 +1394,9 @@ constexpr int LEAF_MIN_SHARE = 4;
 // Sharing is m S / (T 2^L) queries per (tree, leaf): m / 2^L for one leaf per tree, and for the
 // priority search with S leaves a query as many as its budget spreads over the forest's leaves.
 // The priority search's small leaves (the paper's p of a few dozen points) pair up in the
-// tensor-core kernel's row tiles (at 10^6 x 960, p = 64, c = 512: 37.3 ms against 45.7 ms for the
-// streaming kernel per 10^4 queries, bf16); the float32 kernel's 256-row tiles would stay mostly
-// empty there, so float32 priority searches remain with the streaming kernel.
+// tensor-core kernel's row tiles (at 10^6 x 960, p = 64, c = 512: 19.6 ms against 42.4 ms for the
+// streaming kernel per 10^4 queries, bf16).  Float32 priority searches stay with the per-query paths:
+// their distances there are the streaming kernel's bit for bit.
 bool gf_leaf_preferred(const gf_forest *F, int64_t m, int32_t k, int32_t precision, int32_t R, const QueryExtra &x) {
     if (x.leaf_budget > 0 && precision == GF_FP32) return false;
     const int64_t S = x.leaf_budget > 0 ? x.leaf_budget : F->T;
