@@ -210,9 +210,13 @@ __device__ __forceinline__ void var_accum(const BuildParams &P, int tree, const 
     }
 }
 
+// Sums beyond float32's range (a spread above some 1e19) give infinities or NaN: such a variance counts
+// as +inf, so that the rankings below compare values of a total order.  (With NaN among them the lanes of
+// a ranking warp disagree on the winner and run out of dimensions.)
 __device__ __forceinline__ double var_of(double S1, double S2, long long c) {
     if (c < 2) return 0.0;
-    return (S2 - S1 * S1 / (double)c) / (double)(c - 1);
+    const double v = (S2 - S1 * S1 / (double)c) / (double)(c - 1);
+    return v == v ? v : __longlong_as_double(0x7ff0000000000000ll);
 }
 
 __device__ __forceinline__ bool better(double va, int da, double vb, int db) {
