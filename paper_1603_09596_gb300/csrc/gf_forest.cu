@@ -465,13 +465,16 @@ __global__ void __launch_bounds__(256) k_to_fp8(const float *__restrict__ x, int
             unsigned w[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const float f[4] = {v[u].x * inv, v[u].y * inv, v[u].z * inv, v[u].w * inv};
+                // (zeros past d: 0 * inv is NaN where 448 / a overflows)
+                const int c = j + 4 * u;
+                const float f[4] = {c < d ? v[u].x * inv : 0.f, c + 1 < d ? v[u].y * inv : 0.f,
+                                    c + 2 < d ? v[u].z * inv : 0.f, c + 3 < d ? v[u].w * inv : 0.f};
                 w[u] = 0;
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
-                    const __nv_fp8_storage_t c = __nv_cvt_float_to_fp8(f[h], __NV_SATFINITE, __NV_E4M3);
-                    w[u] |= (unsigned)c << (8 * h);
-                    const __half_raw hr = __nv_cvt_fp8_to_halfraw(c, __NV_E4M3);
+                    const __nv_fp8_storage_t code = __nv_cvt_float_to_fp8(f[h], __NV_SATFINITE, __NV_E4M3);
+                    w[u] |= (unsigned)code << (8 * h);
+                    const __half_raw hr = __nv_cvt_fp8_to_halfraw(code, __NV_E4M3);
                     sum.add(__half2float(*reinterpret_cast<const __half *>(&hr)));
                 }
             }
