@@ -313,7 +313,11 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 // a step, plus the float32 rounding of x - low_j, of the product and of 1 / s_j against s_j, together
 // under 0.02 of a step at 65,000 steps), so over a node of c points the square root of
 // the sum of squared deviations moves by at most QERR sqrt(c) s_j (triangle inequality), which bounds
-// the variance on both sides.  A level's sums read 2 bytes a coordinate instead of 4 and cost a few
+// the variance on both sides.  What has to lie between the bounds is the variance as the full sums give
+// it.  Over the up to 8192 points they add at a time, these are off by some 2^-38 of range_j^2 a point,
+// a sixtieth of s_j^2 (ROUNDED allows half of it), as long as nothing under- or overflows: for range_j
+// in [QLOW, QHIGH].  Below, squares may vanish, but the sums stay at most c (range_j^2 + 2^-147): no
+// lower bound, that upper one.  Above, nothing is known.  A level's sums read 2 bytes a coordinate instead of 4 and cost a few
 // integer instructions instead of some 26 of compensated float32: 500,000 x 960, T = 32, a level took
 // 15.4 ms of compensated sums (1.0e12 coordinates/s, bound by those instructions) and takes 2.1 ms of
 // k_qsum over half the points (7.4 TB/s of rows: HBM) and 0.8 ms of k_exact; the build with its bf16
@@ -321,6 +325,8 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 constexpr int CAND_MAX = 64;       // dimensions listed per node; -1: more, the node is summed in full
 constexpr float QERR = 0.52f;
 constexpr float QSTEPS = 65000.f;  // s_j = range_j / QSTEPS
+constexpr float QLOW = 1e-12f, QHIGH = 1e14f;  // s_j^2 2^-24 and 2^31 range_j^2 are normal floats
+constexpr float ROUNDED = 0.5f;
 constexpr int QBIAS = 32500;       // half of them
 constexpr int QCHUNK = 2048;       // points a CTA sums
 constexpr long long QSUM_BYTES = 1ll << 30;  // sums kept for a level's nodes (and its parents')
@@ -346,8 +352,8 @@ __global__ void __launch_bounds__(256) k_range(const float *__restrict__ x, long
     atomicMax(rng + d + j, range_bits(hi));
 }
 
-// qdim[j] = (low, 1 / s, s); s = 0: a constant dimension; s < 0: a range outside [1e-30, 1e30], whose
-// variance is left unknown (every q the same)
+// qdim[j] = (low, 1 / s, s); s = 0: a constant dimension; s = -range: one below QLOW; s = +inf: one above
+// QHIGH (every q the same in these three)
 __global__ void k_qdim(const unsigned *__restrict__ rng, int d, float4 *qdim) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= d) return;
@@ -355,8 +361,8 @@ __global__ void k_qdim(const unsigned *__restrict__ rng, int d, float4 *qdim) {
     const float range = hi - lo;
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
     if (range != 0.f) {
-        if (range >= 1e-30f && range <= 1e30f) q = make_float4(lo, QSTEPS / range, range / QSTEPS, 0.f);
-        else q.z = -1.f;
+        if (range >= QLOW && range <= QHIGH) q = make_float4(lo, QSTEPS / range, range / QSTEPS, 0.f);
+        else q.z = range < QLOW ? -range : __int_as_float(0x7f800000);
     }
     qdim[j] = q;
 }
@@ -477,18 +483,18 @@ __global__ void __launch_bounds__(256) k_qsum(BuildParams P, int l, int mode, lo
 
 // Bounds of one dimension's sum of squared deviations over a node of c points, in units of
 // (c - 1) x variance, from the sums of q and q^2: evaluated in float32 with room for its rounding
-// (2^-20 of the second moment, 1e-5 of the result).
+// (2^-20 of the second moment, 1e-5 of the result) and for the full sums' own.
 __device__ __forceinline__ void dev_bounds(long long S1, long long S2, float c, float s, float &lo, float &hi) {
-    if (s < 0.f) {
+    if (s < 0.f || s > QHIGH) {
         lo = 0.f;
-        hi = __int_as_float(0x7f800000);
+        hi = s < 0.f ? c * (s * s * 1.001f + 1e-37f) : __int_as_float(0x7f800000);
         return;
     }
     const float m2 = (float)S2, m1 = (float)S1;
-    const float v = m2 - m1 * (m1 / c), e = m2 * 9.5367431640625e-7f, h = QERR * sqrtf(c);
-    const float rl = fmaxf(sqrtf(fmaxf(v - e, 0.f)) - h, 0.f) * s, rh = s == 0.f ? 0.f : (sqrtf(fmaxf(v + e, 0.f)) + h) * s;
-    lo = rl * rl * (1.f - 1e-5f);
-    hi = rh * rh * (1.f + 1e-5f);
+    const float v = m2 - m1 * (m1 / c), e = m2 * 9.5367431640625e-7f, h = QERR * sqrtf(c), s2 = s * s;
+    const float rl = fmaxf(sqrtf(fmaxf(v - e, 0.f)) - h, 0.f), rh = sqrtf(fmaxf(v + e, 0.f)) + h;
+    lo = fmaxf(rl * rl - ROUNDED * c, 0.f) * s2 * (1.f - 1e-5f);
+    hi = (rh * rh + ROUNDED * c) * s2 * (1.f + 1e-5f);
 }
 
 // The dimensions that may be among the t of largest variance, per node: those whose upper bound

@@ -31,3 +31,38 @@ def test_variances_beyond_float32_count_as_equal_largest(gf, form, n, d, T, p):
     for tree in range(T):
         assert F.split_dim[tree].tolist() == [oracle.node_draw(3, tree, j) % 5 for j in range(F.split_dim.shape[1])]
     check_forest(F, X, 5, 3, 1, 0, check_dims=False)
+
+
+def ramp(X):    # dimensions of every size at which squares of float32 vanish, pair by pair of columns
+    return X * (10.0 ** np.linspace(-26, -9, X.shape[1])).astype(np.float32)
+
+
+def steep(X):   # from vanishing squares to overflowing ones
+    return X * (10.0 ** np.linspace(-30, 30, X.shape[1])).astype(np.float32)
+
+
+def speck(X):   # ordinary points, one dimension in three far below them, one dimension far above
+    X[:, ::3] *= np.float32(1e-22)
+    X[:, 7] *= np.float32(1e13)
+    return X
+
+
+def faint(X):   # equal spreads, at which float32 keeps a few bits of the squares
+    return (np.random.default_rng(X.shape[0]).standard_normal(X.shape) * 1e-22).astype(np.float32)
+
+
+SCALES = [1e-12, 1e-15, 1e-18, 1e-20, 1e-22, 1e-26, 1e-37, 1e15, 1e19]
+
+
+@pytest.mark.parametrize("change", SCALES + [ramp, steep, speck, faint])
+@pytest.mark.parametrize("n,d,T,p", [(9001, 90, 2, 300), (2500, 101, 3, 20), (3000, 40, 2, 30)])
+def test_fixed_point_bounds_hold_where_squares_leave_float32(gf, change, n, d, T, p):
+    """Reflections by the zero vector leave the points as they are and the build without the bounds: it
+    sums every dimension, and the forest has to be that one, node for node."""
+    X, _ = synth.mixture(n, d, 1, "B", seed=n + d)
+    X = np.ascontiguousarray(change(X) if callable(change) else X * np.float32(change))
+    _, A = gpu_build(gf, X, T, p, t=5, seed=4)
+    _, B = gpu_build(gf, X, T, p, t=5, seed=4, U=np.zeros((T, d), np.float32))
+    assert np.array_equal(A.split_dim, B.split_dim)
+    assert np.array_equal(A.split_val, B.split_val)
+    assert np.array_equal(A.perm, B.perm)
