@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <unordered_map>
 #include <vector>
 
 // ---------------------------------------------------------------- errors
@@ -74,6 +75,31 @@ extern "C" void gf_query_opts_default(gf_query_opts *o) {
     if (!o) return;
     std::memset(o, 0, sizeof *o);
     o->precision = GF_FP32;
+}
+
+// ---------------------------------------------------------------- shared memory limits
+
+cudaError_t gf_smem_limit(const void *kern, size_t smem) {
+    static std::mutex mu;
+    static std::unordered_map<const void *, size_t> fixed;  // kernel -> its static shared memory
+    if (smem <= 32 * 1024) return cudaSuccess;  // within the default 48 KB beside any kernel's static share
+    int dev = 0, all = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    size_t own = 0;
+    {
+        std::lock_guard<std::mutex> g(mu);
+        auto it = fixed.find(kern);
+        if (it == fixed.end()) {
+            cudaFuncAttributes fa;
+            if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+            it = fixed.emplace(kern, fa.sharedSizeBytes).first;
+        }
+        own = it->second;
+    }
+    if (own + smem > (size_t)all) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, all - (int)own);
 }
 
 // ---------------------------------------------------------------- per-call scratch

@@ -120,6 +120,12 @@ int gf_cuda_fail(cudaError_t e, const char *what);
 // Allocation with the library's error code (nothing is leaked on failure).
 int gf_dmalloc(void **p, size_t bytes);
 
+// Lets a kernel be launched with `smem` bytes of dynamic shared memory.  The limit is the kernel's, for all
+// threads of the process, so every launch sets the same one: all that the device has beside the kernel's
+// static shared memory.  (Set to each launch's own size, one thread's launch could find it lowered by
+// another's.)  cudaErrorInvalidValue: more than there is.
+cudaError_t gf_smem_limit(const void *kern, size_t smem);
+
 // ---------------------------------------------------------------- entry points between units
 
 // Forest storage (gf_forest.cu).  gf_forest_alloc: shape fields and storage of x / nodes / perm;

@@ -1535,8 +1535,7 @@ int gf_launch_leaf(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
 #define GF_MERGE(NCV)                                                                                    \
     if (ncf == NCV) {                                                                                    \
         auto kern = small ? k_leaf_merge<NCV, true> : k_leaf_merge<NCV, false>;                          \
-        if (msmem > 46 * 1024 &&                                                                         \
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem)) != cudaSuccess) \
+        if ((e = gf_smem_limit((const void *)kern, msmem)) != cudaSuccess)                               \
             return fail(e, "cudaFuncSetAttribute(k_leaf_merge)");                                        \
         kern<<<mg, small ? 128 : 256, msmem, st>>>(view_of(F), Q, m, k, R, S, !f32, slots, part, tau, (long long *)ids, dists); \
     }

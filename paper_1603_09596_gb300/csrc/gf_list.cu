@@ -624,10 +624,8 @@ cudaError_t launch_admit_d(const gf_forest *F, const float *Q, const Leaves &V, 
                          const ListPlan &P, unsigned long long *keys, int *cnt, cudaStream_t st) {
     auto kern = k_list_admit<BITS, SHORT, NT, DESC>;
     const size_t smem = (size_t)P.words * 4;
-    if (smem > 40 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = gf_smem_limit((const void *)kern, smem);
+    if (e != cudaSuccess) return e;
     if (DESC) {  // the call's first launch
         kern<<<(unsigned)nq, NT, smem, st>>>(view_of(F), Q, V, q0, order, P.words, P.cap, keys, cnt);
         return cudaGetLastError();
@@ -654,10 +652,8 @@ cudaError_t launch_score(const gf_forest *F, const float *Q, long long q0, long 
     const int parts = (P.cap + B - 1) / B;
     const size_t smem = (size_t)ldq_of(F->d) * 4 + (size_t)B * 4;
     auto kern = k_list_score<PREC, NC, G>;
-    if (smem > 40 * 1024) {  // (beside a few KB of static shared memory)
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = gf_smem_limit((const void *)kern, smem);
+    if (e != cudaSuccess) return e;
     return launch_after(kern, nq * parts, 256, smem, st, view_of(F), Q, q0, order, parts, B, P.cap, cnt, keys);
 }
 
@@ -679,10 +675,8 @@ cudaError_t launch_select(const gf_forest *F, const float *Q, long long q0, long
                           int64_t *ids, float *dists, int *ncand_out, cudaStream_t st) {
     const size_t smem = select_smem(F, rerank);
     auto kern = k_list_select<NCF, NT>;
-    if (smem > 40 * 1024) {  // (beside a few KB of static shared memory)
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = gf_smem_limit((const void *)kern, smem);
+    if (e != cudaSuccess) return e;
     return launch_after(kern, nq, NT, smem, st, view_of(F), Q, q0, k, keep, rerank, order, P.cap, cnt, keys, (long long *)ids,
                         dists, ncand_out);
 }
@@ -700,10 +694,8 @@ cudaError_t launch_one(const gf_forest *F, const float *Q, int64_t m, int k, int
                        int *ncand_out, cudaStream_t st) {
     auto kern = k_list_one<PREC, NC, NCF, NC == 1 ? 8 : NC == 2 ? 4 : 2>;
     const size_t smem = one_smem(F);
-    if (smem > 40 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = gf_smem_limit((const void *)kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<(unsigned)m, 256, smem, st>>>(view_of(F), Q, k, keep, one_words(F), (long long *)ids, dists, ncand_out);
     return cudaGetLastError();
 }
@@ -798,8 +790,7 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     if (m >= ORDER_MIN && x.order != GF_ORDER_GIVEN) {
         order = (int *)(ws + P.order);
         const size_t os = (size_t)4 << std::min(F->L, ORDER_BITS);
-        if (os > 40 * 1024 && (e = cudaFuncSetAttribute(k_list_order, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os)) != cudaSuccess)
-            return fail(e, "cudaFuncSetAttribute(k_list_order)");
+        if ((e = gf_smem_limit((const void *)k_list_order, os)) != cudaSuccess) return fail(e, "k_list_order's shared memory");
         k_list_order<<<1, 1024, os, st>>>(V, F->L, m, order);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "k_list_order launch");
     }

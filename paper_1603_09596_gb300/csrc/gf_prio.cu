@@ -299,8 +299,7 @@ int launch_prio(const gf_forest *F, const float *Q, int64_t m, int budget, unsig
     const int warps = (int)std::min<size_t>(PRIO_WARPS, (size_t)lim / per_warp);
     if (warps < 1) return gf_fail(GF_EUNSUPPORTED, "leaf budget %d needs %zu B of shared memory", budget, per_warp);
     const size_t smem = per_warp * warps;
-    if (smem > 48 * 1024)
-        GF_CUDA_TRY(cudaFuncSetAttribute(k_prio_leaves<Place>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GF_CUDA_TRY(gf_smem_limit((const void *)k_prio_leaves<Place>, smem));
     const long long blocks = std::min<long long>((m + warps - 1) / warps, (long long)F->num_sms * 256);
     k_prio_leaves<Place><<<(unsigned)blocks, warps * 32, smem, st>>>(view_of(F), Q, m, budget, leaves, nleaves);
     GF_CUDA_TRY(cudaGetLastError());

@@ -634,11 +634,8 @@ int nc_for(int chunks) {
 
 template <typename KernelT>
 int prep_kernel(KernelT kern, size_t smem) {
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return gf_cuda_fail(e, "cudaFuncSetAttribute(max dynamic smem)");
-    }
-    return GF_OK;
+    const cudaError_t e = gf_smem_limit((const void *)kern, smem);
+    return e == cudaSuccess ? GF_OK : gf_cuda_fail(e, "cudaFuncSetAttribute(max dynamic smem)");
 }
 
 int check_smem(const gf_forest *F, size_t smem) {
@@ -857,10 +854,8 @@ int dispatch_prec(const gf_forest *F, const float *Q, int64_t m, int32_t k, int3
 cudaError_t gf_sort_order(int64_t m, const unsigned long long *okeys, int *order, cudaStream_t st) {
     const long long chunks = (m + ORDER_CHUNK - 1) / ORDER_CHUNK;
     const size_t smem = (size_t)next_pow2((int)std::min<long long>(m, ORDER_CHUNK)) * 8;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_order_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = gf_smem_limit((const void *)k_order_sort, smem);
+    if (e != cudaSuccess) return e;
     k_order_sort<<<(unsigned)chunks, 1024, smem, st>>>(m, okeys, order);
     return cudaGetLastError();
 }
