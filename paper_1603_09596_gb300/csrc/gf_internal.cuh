@@ -189,9 +189,10 @@ const char *gf_leaf_unsupported(const gf_forest *F, int64_t m, int32_t k, int32_
                                 const QueryExtra &x);
 
 // Staged per-query path (gf_list.cu).  usable: its selection and shared memory hold this query.
-// launch: *ran = false (and GF_OK) when its scratch could not be allocated.
+// launch: *ran = false (and GF_OK) when its scratch could not be allocated or is better not (sorts: the sort
+// kernel can answer the call).
 bool gf_list_usable(const gf_forest *F, int64_t m, int32_t k, int32_t precision, int32_t R, const QueryExtra &x);
-int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision, int32_t R,
+int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision, int32_t R, bool sorts,
                    cudaStream_t st, int64_t *ids, float *dists, const QueryExtra &x, bool *ran);
 // order[0..m) = the queries of okeys (leaf << 32 | query) sorted, in chunks of 16,384
 cudaError_t gf_sort_order(int64_t m, const unsigned long long *okeys, int *order, cudaStream_t st);

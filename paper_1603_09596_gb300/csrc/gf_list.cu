@@ -737,7 +737,18 @@ bool gf_list_usable(const gf_forest *F, int64_t m, int32_t k, int32_t precision,
     return (size_t)ldq_of(F->d) * 4 + 256 * 4 <= lim && select_smem(F, true) + 4096 <= lim;
 }
 
-int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision, int32_t R,
+namespace {
+
+// Whether work on st goes into a graph.
+bool captured(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) cudaGetLastError();
+    return status != cudaStreamCaptureStatusNone;
+}
+
+}  // namespace
+
+int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision, int32_t R, bool sorts,
                    cudaStream_t st, int64_t *ids, float *dists, const QueryExtra &x, bool *ran) {
     *ran = false;
     const bool prio = x.leaf_budget > 0, rerank = precision != GF_FP32;
@@ -752,6 +763,9 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
         if (e == cudaSuccess) e = gf_record(x, 1, st);
         return e == cudaSuccess ? GF_OK : gf_cuda_fail(e, "k_list_one launch");
     }
+    // In a graph the scratch would be an allocation node, and such a graph has one instance at a time and
+    // cannot be a node of another: a call that the sort kernel can answer stays with it, which needs none.
+    if (sorts && captured(st)) return GF_OK;
     const ListPlan P = list_plan(F, m, x.leaf_budget);
     char *ws = nullptr;
     if (gf_scratch_alloc((void **)&ws, P.total, st) != cudaSuccess) {

@@ -817,6 +817,13 @@ int stream_grid_prec(const gf_forest *F, int64_t m, int k, int R, int warps, int
     return gf_fail(GF_EUNSUPPORTED, "no kernel for chunk classes %d/%d", nc, ncf);
 }
 
+// The one-CTA kernel of a search of one leaf per tree: the caller's choice, or sort while the candidates
+// and the query fit well beside a second CTA.
+int one_cta_algo(const gf_forest *F, const QueryExtra &x) {
+    if (x.algo != GF_ALGO_AUTO) return x.algo;
+    return F->cand_cap <= 4096 && smem_bytes(F->d, F->T, F->cand_cap) <= 100 * 1024 && !x.ncand_out ? GF_ALGO_SORT : GF_ALGO_STREAM;
+}
+
 template <int PREC>
 int dispatch_prec(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t R, int warps,
                   int cps, cudaStream_t st, int64_t *ids, float *dists, const QueryExtra &x) {
@@ -828,10 +835,7 @@ int dispatch_prec(const gf_forest *F, const float *Q, int64_t m, int32_t k, int3
         if (algo == GF_ALGO_SORT) return gf_fail(GF_EINVAL, "the priority search runs in the streaming kernel only");
         algo = GF_ALGO_STREAM;
     }
-    if (algo == GF_ALGO_AUTO) {
-        const size_t sort_smem = smem_bytes(F->d, F->T, F->cand_cap);
-        algo = (F->cand_cap <= 4096 && sort_smem <= 100 * 1024 && !x.ncand_out) ? GF_ALGO_SORT : GF_ALGO_STREAM;
-    }
+    if (algo == GF_ALGO_AUTO) algo = one_cta_algo(F, x);
     if (algo == GF_ALGO_SORT && x.ncand_out)
         return gf_fail(GF_EINVAL, "candidate counts are reported by the streaming kernel only");
 #define GF_CASE(A, B)                                                                              \
@@ -871,7 +875,8 @@ int gf_launch_query(const gf_forest *F, const float *Q, int64_t m, int32_t k, in
     }
     if (x.algo == GF_ALGO_AUTO && !x.shaped && gf_list_usable(F, m, k, precision, R, x)) {
         bool ran = false;
-        const int r = gf_launch_list(F, Q, m, k, precision, R, st, ids, dists, x, &ran);
+        const bool sorts = x.leaf_budget <= F->T && one_cta_algo(F, x) == GF_ALGO_SORT;
+        const int r = gf_launch_list(F, Q, m, k, precision, R, sorts, st, ids, dists, x, &ran);
         if (r || ran) return r;
     }
     switch (precision) {

@@ -1,0 +1,68 @@
+"""Which kernels GF_ALGO_AUTO takes, by what that means for the caller."""
+import ctypes as C
+
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gf():
+    import paper_1603_09596_gb300 as g
+    g.lib()
+    return g
+
+
+def cudart():
+    for name in ("libcudart.so.13", "libcudart.so"):
+        try:
+            return C.CDLL(name)
+        except OSError:
+            pass
+    pytest.skip("the CUDA runtime cannot be opened by name")
+
+
+# calls within the sort kernel's reach: the staged steps', and the single launch's
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8"])
+@pytest.mark.parametrize("n,d,T,p,m", [(10_000, 960, 16, 64, 100), (50_000, 512, 16, 256, 27), (10_000, 128, 8, 32, 100)])
+def test_small_calls_are_captured_without_memory_nodes(gf, prec, n, d, T, p, m):
+    """Two instances of the captured graph live side by side and give the uncaptured call's answers: a
+    graph that allocates can have only one."""
+    rt = cudart()
+    X, Q = synth.mixture(n, d, m, "B", seed=81, qseed=82)
+    F = gf.gf_build(torch.from_numpy(X).cuda(), T, p, seed=1)
+    P, R = gf.PRECISIONS[prec], 0 if prec == "fp32" else 32
+    if P:
+        gf.gf_forest_add_screen(F, P)
+    Qg = torch.from_numpy(Q).cuda()
+    want = gf.gf_query(F, Qg, 10, precision=P, rerank_R=R, algo=gf.GF_ALGO_SORT)
+    out = (torch.empty_like(want[0]), torch.empty_like(want[1]))
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = C.c_void_p()
+    st = C.c_void_p(s.cuda_stream)
+    assert rt.cudaStreamBeginCapture(st, 2) == 0  # relaxed
+    try:
+        gf.gf_query(F, Qg, 10, precision=P, rerank_R=R, out=out, stream=s)
+    finally:
+        assert rt.cudaStreamEndCapture(st, C.byref(graph)) == 0
+    instances = []
+    try:
+        for _ in range(2):
+            h = C.c_void_p()
+            assert rt.cudaGraphInstantiate(C.byref(h), graph, C.c_ulonglong(0)) == 0
+            instances.append(h)
+        for h in instances:
+            out[0].zero_()
+            torch.cuda.synchronize()
+            assert rt.cudaGraphLaunch(h, st) == 0
+            torch.cuda.synchronize()
+            assert torch.equal(out[0], want[0]) and torch.equal(out[1], want[1])
+    finally:
+        rt.cudaGetLastError()
+        for h in instances:
+            rt.cudaGraphExecDestroy(h)
+        rt.cudaGraphDestroy(graph)
