@@ -715,6 +715,10 @@ cudaError_t one_prec(const gf_forest *F, const float *Q, int64_t m, int k, int k
     return cudaErrorInvalidValue;
 }
 
+int row_bytes(const gf_forest *F, int32_t precision) {
+    return 16 * (precision == GF_FP32 ? chunks_of<P_F32>(F) : precision == GF_BF16_RERANK ? chunks_of<P_BF16>(F) : chunks_of<P_FP8>(F));
+}
+
 // One launch for the whole call: few candidates a query, rows of at most 4 KB, no reflections, little
 // to score in all, and either little for one CTA (its rows come at some 50 GB/s) or about a CTA an SM.
 // Microseconds a call, one launch / the staged steps: 640 candidates of 1 KB, m = 10: 23 / 32, 304:
@@ -722,8 +726,24 @@ cudaError_t one_prec(const gf_forest *F, const float *Q, int64_t m, int k, int k
 // 160 of 512 bytes, m = 100: 20 / 33, 1000: 25 / 50 (of which the host's part was about 19; now 13).
 bool one_launch(const gf_forest *F, int64_t m, int32_t precision, const QueryExtra &x) {
     if (x.leaf_budget > 0 || F->U || F->cand_cap > SEL_BUF || nc_of(F->ldx / 4) == 0 || m * F->cand_cap > ONE_MAX) return false;
-    const int chunks = precision == GF_FP32 ? chunks_of<P_F32>(F) : precision == GF_BF16_RERANK ? chunks_of<P_BF16>(F) : chunks_of<P_FP8>(F);
-    return (int64_t)F->cand_cap * chunks * 16 <= ONE_BYTES || m >= F->num_sms;
+    return (int64_t)F->cand_cap * row_bytes(F, precision) <= ONE_BYTES || m >= F->num_sms;
+}
+
+// Whether a call that the sort kernel can answer is better left to it: few candidates a query, so that
+// neither the staged steps' launches nor the single launch's eight warps a query pay.  Fitted to 1,400
+// searches of 200 to 500,000 points, T = 1 to 64, at most 4096 candidates, 1 to 30,000 queries, every
+// precision: the staged steps or the single launch were the slower ones in 148 (down to 0.56 of the
+// sort kernel's speed), nearly all of them here; 14 remain (down to 0.81).  Microseconds, this path /
+// sort kernel: single launch, leaves of 2, T = 62, m = 1151: 48 / 27; 1, T = 1, m = 2155: 44 / 31; staged,
+// 6 candidates of 5.4 KB, m = 11: 22 / 14; 82 of 6 KB (k = 128), m = 551: 50 / 30; 34 of 20 bytes, m = 10,704:
+// 150 / 114.
+bool few_candidates(const gf_forest *F, int64_t m, int keep, int32_t precision, bool one) {
+    const int leaf = F->max_leaf, cap = F->cand_cap, row = row_bytes(F, precision);
+    if (one)
+        return (row <= 1024 && ((leaf <= 8 && F->T >= 12 && m * F->T >= 4096) || (leaf <= 3 && F->T >= 32))) ||
+               (row <= 512 && cap <= 8 && m >= 1024);
+    const bool few = m * cap <= 4096 || row >= 4096;
+    return (leaf <= 3 && (few || row <= 1024)) || ((cap <= 96 || cap <= keep) && few) || (cap <= 128 && row <= 512);
 }
 
 }  // namespace
@@ -753,7 +773,9 @@ int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int
     *ran = false;
     const bool prio = x.leaf_budget > 0, rerank = precision != GF_FP32;
     const int keep = rerank ? R : k;
-    if (one_launch(F, m, precision, x)) {
+    const bool one = one_launch(F, m, precision, x);
+    if (sorts && few_candidates(F, m, keep, precision, one)) return GF_OK;
+    if (one) {
         *ran = true;
         cudaError_t e = gf_record(x, 0, st);
         if (e == cudaSuccess)

@@ -66,3 +66,27 @@ def test_small_calls_are_captured_without_memory_nodes(gf, prec, n, d, T, p, m):
         for h in instances:
             rt.cudaGraphExecDestroy(h)
         rt.cudaGraphDestroy(graph)
+
+
+# (n, d, T, p, m, k): on both sides of the lines between the sort kernel and the staged path or the single
+# launch: leaves of 2 to 9 points, 8 and 9 candidates, 96 and 97, fewer than k and more, short rows and long
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8"])
+@pytest.mark.parametrize("n,d,T,p,m,k", [
+    (4217, 26, 40, 3, 300, 5), (4217, 26, 12, 9, 400, 5), (512, 300, 12, 8, 400, 5), (4000, 128, 4, 2, 1100, 3),
+    (900, 128, 9, 1, 1100, 3), (3072, 1100, 8, 12, 40, 10), (3104, 1100, 1, 97, 50, 10), (5000, 2200, 6, 20, 30, 128),
+    (3000, 5, 20, 3, 9000, 2), (30_000, 60, 4, 32, 6000, 33), (2000, 1500, 4, 1, 3, 1),
+])
+def test_routes_of_few_candidates_answer_alike(gf, prec, n, d, T, p, m, k):
+    X, Q = synth.mixture(n, d, m, "B", seed=83, qseed=84)
+    F = gf.gf_build(torch.from_numpy(X).cuda(), T, p, t=min(5, d), seed=1)
+    P, R = gf.PRECISIONS[prec], 0 if prec == "fp32" else max(k, 40)  # (no leaf-major batch at 40)
+    if P:
+        gf.gf_forest_add_screen(F, P)
+    Qg = torch.from_numpy(Q).cuda()
+    for order in (gf.GF_ORDER_AUTO, gf.GF_ORDER_GIVEN):
+        a = gf.gf_query(F, Qg, k, precision=P, rerank_R=R, order=order)
+        if prec == "fp32" and k <= 32 and m >> F.info.L >= 4:  # leaf-major: another order of additions
+            continue
+        for algo in (gf.GF_ALGO_SORT, gf.GF_ALGO_STREAM):
+            b = gf.gf_query(F, Qg, k, precision=P, rerank_R=R, algo=algo)
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
