@@ -329,6 +329,9 @@ constexpr float QLOW = 1e-12f, QHIGH = 1e14f;  // s_j^2 2^-24 and 2^31 range_j^2
 constexpr float ROUNDED = 0.5f;
 constexpr int QBIAS = 32500;       // half of them
 constexpr int QCHUNK = 2048;       // points a CTA sums
+// Points from which a build takes the fixed-point pass (ms without / with it, d = 128, T = 8: 1000 points
+// 0.67 / 0.66, 2048 1.09 / 1.03, 5000 2.54 / 1.96; below, its launches and memory cost up to 0.1 ms).
+constexpr long long QMIN = 2048;
 constexpr long long QSUM_BYTES = 1ll << 30;  // sums kept for a level's nodes (and its parents')
 
 __device__ __forceinline__ unsigned range_bits(float f) {
@@ -1052,7 +1055,13 @@ struct DevBuf {
 // Scratch of the fixed-point pass (k_qsum and after); without it the build takes the full-precision
 // sums of every dimension.
 struct QuantScratch {
-    DevBuf rng, qdim, xq, sums[2], ncand, cand, segs, xpart;
+    DevBuf mem;             // all of it (nine allocations and frees took 0.1 ms, half of a build of 300 points)
+    unsigned *rng = nullptr;
+    float4 *qdim = nullptr;
+    short *xq = nullptr;
+    long long *sums[2] = {nullptr, nullptr};
+    int *ncand = nullptr, *cand = nullptr, *segs = nullptr;
+    double *xpart = nullptr;
     int ldq = 0, tpr = 8;
     long long cap = 0;      // nodes each sums buffer holds
     bool on = false;
@@ -1065,20 +1074,35 @@ cudaError_t quant_prepare(QuantScratch &S, const BuildParams &P, long long wides
     S.ldq = (d + 7) / 8 * 8;
     while (S.tpr < 128 && S.tpr * 8 < d) S.tpr <<= 1;
     S.cap = std::max(1ll, std::min(widest, QSUM_BYTES / (16ll * d)));
-    S.on = S.rng.spare((size_t)d * 8) && S.qdim.spare((size_t)d * 16) && S.xq.spare((size_t)P.n * S.ldq * 2) &&
-           S.sums[0].spare((size_t)S.cap * d * 16) && S.sums[1].spare((size_t)S.cap * d * 16) &&
-           S.ncand.spare((size_t)widest * 4) && S.cand.spare((size_t)widest * CAND_MAX * 4) &&
-           S.segs.spare((size_t)widest * 4) && S.xpart.spare((size_t)std::max(1ll, maxch) * 2 * CAND_MAX * 8);
+    size_t total = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t rng = place((size_t)d * 8), qdim = place((size_t)d * 16), xq = place((size_t)P.n * S.ldq * 2);
+    const size_t sums[2] = {place((size_t)S.cap * d * 16), place((size_t)S.cap * d * 16)};
+    const size_t ncand = place((size_t)widest * 4), cand = place((size_t)widest * CAND_MAX * 4), segs = place((size_t)widest * 4);
+    const size_t xpart = place((size_t)maxch * 2 * CAND_MAX * 8);
+    S.on = S.mem.spare(total);
     if (!S.on) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(S.rng.p, 0xff, (size_t)d * 4, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync((unsigned *)S.rng.p + d, 0, (size_t)d * 4, st);
+    char *m = (char *)S.mem.p;
+    S.rng = (unsigned *)(m + rng);
+    S.qdim = (float4 *)(m + qdim);
+    S.xq = (short *)(m + xq);
+    for (int i = 0; i < 2; ++i) S.sums[i] = (long long *)(m + sums[i]);
+    S.ncand = (int *)(m + ncand);
+    S.cand = (int *)(m + cand);
+    S.segs = (int *)(m + segs);
+    S.xpart = (double *)(m + xpart);
+    cudaError_t e = cudaMemsetAsync(S.rng, 0xff, (size_t)d * 4, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(S.rng + d, 0, (size_t)d * 4, st);
     if (e != cudaSuccess) return e;
     const int rows = 256;
-    k_range<<<dim3((unsigned)((P.n + rows - 1) / rows), (d + 255) / 256), 256, 0, st>>>(P.x, P.n, d, P.ldx, rows, (unsigned *)S.rng.p);
-    k_qdim<<<(d + 255) / 256, 256, 0, st>>>((const unsigned *)S.rng.p, d, (float4 *)S.qdim.p);
+    k_range<<<dim3((unsigned)((P.n + rows - 1) / rows), (d + 255) / 256), 256, 0, st>>>(P.x, P.n, d, P.ldx, rows, S.rng);
+    k_qdim<<<(d + 255) / 256, 256, 0, st>>>(S.rng, d, S.qdim);
     const int dblocks = (S.ldq + S.tpr * 8 - 1) / (S.tpr * 8);
-    k_quant<<<dim3((unsigned)(sms * 8), dblocks), 256, 0, st>>>(P.x, P.n, d, P.ldx, S.ldq, S.tpr, (const float4 *)S.qdim.p,
-                                                              (short *)S.xq.p);
+    k_quant<<<dim3((unsigned)(sms * 8), dblocks), 256, 0, st>>>(P.x, P.n, d, P.ldx, S.ldq, S.tpr, S.qdim, S.xq);
     return cudaGetLastError();
 }
 
@@ -1089,17 +1113,15 @@ cudaError_t quant_level(QuantScratch &S, const BuildParams &P, int l, const int 
     const int nch = (int)((cm + QCHUNK - 1) / QCHUNK);
     const int dblocks = (S.ldq + S.tpr * 8 - 1) / (S.tpr * 8);
     const size_t smem = (size_t)2 * S.tpr * 8 * 8;
-    long long *sums = (long long *)S.sums[l & 1].p, *parent = (long long *)S.sums[(l & 1) ^ 1].p;
+    long long *sums = S.sums[l & 1], *parent = S.sums[(l & 1) ^ 1];
     auto qsum = [&](int mode, long long node0, long long nodes, long long slots) {
         cudaError_t e = nch > 1 ? cudaMemsetAsync(sums, 0, (size_t)slots * P.d * 16, st) : cudaSuccess;
         if (e != cudaSuccess) return e;
-        k_qsum<<<dim3((unsigned)(nodes * nch), dblocks), 256, smem, st>>>(P, l, mode, node0, nch, S.tpr, seq,
-                                                                          (const short *)S.xq.p, S.ldq, sums);
+        k_qsum<<<dim3((unsigned)(nodes * nch), dblocks), 256, smem, st>>>(P, l, mode, node0, nch, S.tpr, seq, S.xq, S.ldq, sums);
         return cudaGetLastError();
     };
     auto pick = [&](long long node0, long long nodes, int derive) {
-        k_cand<<<(unsigned)nodes, NT, 0, st>>>(P, l, node0, derive, (const float4 *)S.qdim.p, parent, sums, (int *)S.ncand.p,
-                                               (int *)S.cand.p);
+        k_cand<<<(unsigned)nodes, NT, 0, st>>>(P, l, node0, derive, S.qdim, parent, sums, S.ncand, S.cand);
         return cudaGetLastError();
     };
     cudaError_t e = cudaSuccess;
@@ -1177,8 +1199,8 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
     GF_CUDA_TRY(cudaFuncSetAttribute(k_level_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_max));
 
     QuantScratch S;
-    if (!F->U && !P.global_scope && L > 0) GF_CUDA_TRY(quant_prepare(S, P, (long long)T << (L - 1), maxch, F->num_sms, st));
-    const int *chosen = S.on ? (const int *)S.ncand.p : nullptr;  // >= 0: the node's split dimension is chosen below
+    if (!F->U && !P.global_scope && L > 0 && n >= QMIN) GF_CUDA_TRY(quant_prepare(S, P, (long long)T << (L - 1), maxch, F->num_sms, st));
+    const int *chosen = S.on ? S.ncand : nullptr;  // >= 0: the node's split dimension is chosen below
 
     const int ndb = (F->d + DB - 1) / DB;
     for (int l = 0; l < L; ++l) {
@@ -1191,10 +1213,9 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
             const bool sel = S.on && l > 0;
             if (sel) {
                 GF_CUDA_TRY(quant_level(S, P, l, bufA, st));
-                k_exact<<<(unsigned)((nseg * 32 + NT - 1) / NT), NT, 0, st>>>(P, l, nseg, bufA, chosen, (const int *)S.cand.p,
-                                                                              (int *)S.segs.p);
+                k_exact<<<(unsigned)((nseg * 32 + NT - 1) / NT), NT, 0, st>>>(P, l, nseg, bufA, chosen, S.cand, S.segs);
             }
-            k_level_small<<<(unsigned)nseg, NT, smem, st>>>(P, l, bufA, sel ? (const int *)S.segs.p : nullptr, chosen, bufB);
+            k_level_small<<<(unsigned)nseg, NT, smem, st>>>(P, l, bufA, sel ? S.segs : nullptr, chosen, bufB);
             GF_CUDA_TRY(cudaGetLastError());
         } else {
             const int nch = (int)((cm + CHUNK - 1) / CHUNK);
@@ -1208,9 +1229,9 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
                     GF_CUDA_TRY(quant_level(S, P, l, bufA, st));
                     const long long own = l == 0 ? nch : nchunks;  // level 0: tree 0's chunks serve all
                     k_exact_chunk<<<(unsigned)((own * 32 + NT - 1) / NT), NT, 0, st>>>(
-                        P, l, nch, own, bufA, chosen, (const int *)S.cand.p, (double *)S.xpart.p);
+                        P, l, nch, own, bufA, chosen, S.cand, S.xpart);
                     k_exact_pick<<<(unsigned)((nseg * 32 + NT - 1) / NT), NT, 0, st>>>(
-                        P, l, nch, nseg, chosen, (const int *)S.cand.p, (const double *)S.xpart.p, seg_s);
+                        P, l, nch, nseg, chosen, S.cand, S.xpart, seg_s);
                 }
                 k_var_partial<<<dim3((unsigned)nchunks, ndb), NT, 0, st>>>(P, l, nch, bufA, chosen, (double *)part.p);
                 k_var_combine<<<(unsigned)nseg, NT, 0, st>>>(P, l, nch, chosen, (const double *)part.p, seg_s);

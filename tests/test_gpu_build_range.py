@@ -66,3 +66,13 @@ def test_fixed_point_bounds_hold_where_squares_leave_float32(gf, change, n, d, T
     assert np.array_equal(A.split_dim, B.split_dim)
     assert np.array_equal(A.split_val, B.split_val)
     assert np.array_equal(A.perm, B.perm)
+
+
+@pytest.mark.parametrize("n", [2, 2047, 2048, 2049])
+def test_builds_around_the_fixed_point_pass_smallest_size(gf, n):
+    X, _ = synth.mixture(n, 70, 1, "B", seed=n)
+    _, A = gpu_build(gf, X, 3, 8, t=5, seed=4)
+    _, B = gpu_build(gf, X, 3, 8, t=5, seed=4, U=np.zeros((3, 70), np.float32))
+    assert np.array_equal(A.split_dim, B.split_dim)
+    assert np.array_equal(A.split_val, B.split_val)
+    assert np.array_equal(A.perm, B.perm)
