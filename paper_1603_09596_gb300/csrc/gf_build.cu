@@ -404,28 +404,68 @@ __global__ void __launch_bounds__(256) k_quant(const float *__restrict__ x, long
     }
 }
 
-// Which nodes of level l a k_qsum launch sums: idx counts them, seg = (tree << l) + a.
-constexpr int Q_LEFT = 0;  // the left child of every node of level l - 1
-constexpr int Q_FROM = 1;  // nodes node0 + idx
+// What a level's kernels do, settled on the device from the level before.
+// On points whose bounds decide few nodes (a far outlier sets the step of its dimension; many dimensions
+// tie) the pass, a quarter of a level's time where no sums are derived, would be spent for nothing.  After
+// a level that left more than three quarters of its nodes undecided only a few nodes of a level are summed,
+// until those are decided again; the host, which reads the outcome of the first level and of such probes,
+// leaves the levels between probes alone.  Milliseconds, every dimension summed / the pass at every level /
+// with this rule, one far outlier: 500,000 x 960, T = 32 166.1 / 187.6 / 169.8; 200,000 x 256, T = 8 27.8 /
+// 31.0 / 29.2; 100,000 x 128, T = 1 4.7 / 5.9 / 5.4.  Two far points that the deep nodes leave behind, 200,000
+// x 256, T = 8: 27.9 / 23.1 / 23.3.
+enum QMode { Q_ALL, Q_LEFT, Q_PROBE, Q_NONE };  // every node, left ones (the right ones are derived), a few, none
 
-__device__ __forceinline__ long long qsum_seg(int mode, int l, long long node0, long long idx) {
-    if (mode == Q_FROM) return node0 + idx;
-    return ((idx >> (l - 1)) << l) + ((idx & ((1ll << (l - 1)) - 1)) << 1);
+constexpr int PROBE = 8;      // nodes a probe sums, but no more points than there are
+constexpr int TALLY = 1024;   // nodes of a level that count (spread over all of them)
+constexpr long long PROBE_OFTEN = 1ll << 28;  // coordinates times trees from which every second level is probed, else every fourth
+
+struct QLevel {
+    int tried, left;  // counted nodes summed, and those left undecided
+    int sums;         // every node's sums are kept for the next level
+};
+
+__host__ __device__ inline bool q_decides(const QLevel &a) { return a.tried > 0 && 4 * a.left <= 3 * a.tried; }
+
+struct QPlan {
+    QLevel *lv;       // [levels], zeroed
+    long long nodes;  // of this level
+    int first, keeps, stride;  // first: no level before; keeps: a sums buffer holds the level; stride: levels between probes
+};
+
+__device__ __forceinline__ QMode q_mode(const QPlan &W, int l) {
+    if (W.first) return Q_ALL;
+    const QLevel a = W.lv[l - 1];
+    if (!q_decides(a)) return l % W.stride == 0 ? Q_PROBE : Q_NONE;
+    return W.keeps && a.sums ? Q_LEFT : Q_ALL;
+}
+
+// Whether seg is one of about `count` nodes spread over a level, from the middle of each stretch: a tree's
+// first node and its last hold the outermost points.
+__device__ __forceinline__ bool q_sampled(const QPlan &W, long long count, long long seg) {
+    const long long step = max(1ll, W.nodes / count);
+    return seg % step == step / 2;
+}
+
+// Whether k_qsum sums node seg.
+__device__ __forceinline__ bool q_takes(const QPlan &W, QMode mode, int l, long long seg) {
+    if (mode == Q_PROBE) return q_sampled(W, min((long long)PROBE, 1ll << l), seg);
+    return mode == Q_ALL || (mode == Q_LEFT && !(seg & 1));
 }
 
 // Sums of q and q^2 over a chunk of a node, per dimension, exact.  tpr threads cover a row 16 bytes
 // (eight values) each, 256 / tpr rows at a time, eight row loads in flight a thread; bound by the
 // rows it reads (one level of 500,000 x 960, T = 32: half the points, 15.4 GB, 2.05 ms).
-// sums[slot][2][d], slot = seg (Q_LEFT) or idx; several chunks a node are added with (integer, so
-// order-independent) atomics to zeroed sums.
-__global__ void __launch_bounds__(256) k_qsum(BuildParams P, int l, int mode, long long node0, int nch, int tpr,
+// sums[seg - node0][2][d]; several chunks a node are added with (integer, so order-independent) atomics to
+// zeroed sums.
+__global__ void __launch_bounds__(256) k_qsum(BuildParams P, QPlan W, int l, long long node0, int nch, int tpr,
                                               const int *__restrict__ pin, const short *__restrict__ xq, int ldq,
                                               long long *sums) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     long long *sh = reinterpret_cast<long long *>(smem_raw);  // [2][8 tpr]
     const long long idx = blockIdx.x / (unsigned)nch;
     const int ci = (int)(blockIdx.x - (unsigned)idx * (unsigned)nch);
-    const long long seg = qsum_seg(mode, l, node0, idx);
+    const long long seg = node0 + idx;
+    if (!q_takes(W, q_mode(W, l), l, seg)) return;
     const NodeGeo g = geo(P, l, seg);
     const long long beg = min(g.lo + (long long)ci * QCHUNK, g.hi), end = nch == 1 ? g.hi : min(beg + QCHUNK, g.hi);
     const int *rows = pin + (size_t)g.tree * P.n;
@@ -475,7 +515,7 @@ __global__ void __launch_bounds__(256) k_qsum(BuildParams P, int l, int mode, lo
         }
         __syncthreads();
     }
-    long long *o = sums + (size_t)(mode == Q_FROM ? idx : seg) * 2 * P.d;
+    long long *o = sums + (size_t)idx * 2 * P.d;
     for (int i = threadIdx.x; i < 2 * tpr * 8; i += 256) {
         const int h = i >= tpr * 8, j = dbase + i - h * tpr * 8;
         if (j >= P.d) continue;
@@ -502,17 +542,26 @@ __device__ __forceinline__ void dev_bounds(long long S1, long long S2, float c, 
 
 // The dimensions that may be among the t of largest variance, per node: those whose upper bound
 // reaches the t-th largest of the threads' largest lower bounds (t dimensions lie at or above that).
-// derive: an odd (right) node's sums are its parent's minus its left sibling's, and are kept.
-// sums[slot], slot = blockIdx.x = seg - node0; ncand[seg] = -1 when there are more than CAND_MAX.
-__global__ void __launch_bounds__(NT) k_cand(BuildParams P, int l, long long node0, int derive,
+// Q_LEFT: an odd (right) node's sums are its parent's minus its left sibling's, and are kept.
+// sums[slot], slot = blockIdx.x = seg - node0; ncand[seg] = -1: undecided, more than CAND_MAX or not summed.
+__global__ void __launch_bounds__(NT) k_cand(BuildParams P, QPlan W, int l, long long node0,
                                              const float4 *__restrict__ qdim, const long long *__restrict__ parent,
                                              long long *sums, int *ncand, int *cand) {
     __shared__ float top[NT];
     __shared__ float tau;
     __shared__ int count;
     const long long seg = node0 + blockIdx.x;
+    const QMode mode = q_mode(W, l);
+    const bool right = mode == Q_LEFT && (seg & 1);
+    if (seg == 0 && threadIdx.x == 0) W.lv[l].sums = W.keeps && mode <= Q_LEFT;
+    if (!right && !q_takes(W, mode, l, seg)) {
+        if (threadIdx.x == 0) ncand[seg] = -1;
+        return;
+    }
     const NodeGeo g = geo(P, l, seg);
     const float c = (float)(g.hi - g.lo);
+    const bool counts = mode == Q_PROBE || q_sampled(W, TALLY, seg);
+    if (counts && threadIdx.x == 0) atomicAdd(&W.lv[l].tried, 1);
     int *out = cand + seg * CAND_MAX;
     if (g.hi - g.lo < 2) {  // every variance is 0: the first t dimensions
         for (int r = threadIdx.x; r < P.t; r += NT) out[r] = r;
@@ -520,7 +569,6 @@ __global__ void __launch_bounds__(NT) k_cand(BuildParams P, int l, long long nod
         return;
     }
     long long *S = sums + (size_t)blockIdx.x * 2 * P.d;
-    const bool right = derive && (seg & 1);
     const long long *up = right ? parent + (size_t)(l == 1 ? 0 : seg >> 1) * 2 * P.d : nullptr;
     const long long *left = S - 2 * (size_t)P.d;
     float best = -1.f;
@@ -556,7 +604,10 @@ __global__ void __launch_bounds__(NT) k_cand(BuildParams P, int l, long long nod
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) ncand[seg] = count <= CAND_MAX ? count : -1;
+    if (threadIdx.x == 0) {
+        ncand[seg] = count <= CAND_MAX ? count : -1;
+        if (counts && count > CAND_MAX) atomicAdd(&W.lv[l].left, 1);
+    }
 }
 
 // One dimension of var_accum over rows[0..cnt), cnt > 0, K the coordinate of krow: lane `lane` of
@@ -1062,10 +1113,14 @@ struct QuantScratch {
     long long *sums[2] = {nullptr, nullptr};
     int *ncand = nullptr, *cand = nullptr, *segs = nullptr;
     double *xpart = nullptr;
+    QLevel *lv = nullptr;
     int ldq = 0, tpr = 8;
     long long cap = 0;      // nodes each sums buffer holds
     bool on = false;
-    int have = -1;          // the level whose nodes' sums are complete in sums[have & 1]
+    int first = -1;         // the first level it was taken for
+    int stride = 1;         // levels between probes
+    bool decides = true;    // as far as the host knows: the last level it read was decided
+    bool takes(int l) const { return on && (decides || l % stride == 0); }
 };
 
 // Allocates it and makes the 16-bit copy of the points.  widest: nodes of the last level.
@@ -1083,7 +1138,7 @@ cudaError_t quant_prepare(QuantScratch &S, const BuildParams &P, long long wides
     const size_t rng = place((size_t)d * 8), qdim = place((size_t)d * 16), xq = place((size_t)P.n * S.ldq * 2);
     const size_t sums[2] = {place((size_t)S.cap * d * 16), place((size_t)S.cap * d * 16)};
     const size_t ncand = place((size_t)widest * 4), cand = place((size_t)widest * CAND_MAX * 4), segs = place((size_t)widest * 4);
-    const size_t xpart = place((size_t)maxch * 2 * CAND_MAX * 8);
+    const size_t xpart = place((size_t)maxch * 2 * CAND_MAX * 8), lv = place(32 * sizeof(QLevel));
     S.on = S.mem.spare(total);
     if (!S.on) return cudaSuccess;
     char *m = (char *)S.mem.p;
@@ -1095,7 +1150,10 @@ cudaError_t quant_prepare(QuantScratch &S, const BuildParams &P, long long wides
     S.cand = (int *)(m + cand);
     S.segs = (int *)(m + segs);
     S.xpart = (double *)(m + xpart);
-    cudaError_t e = cudaMemsetAsync(S.rng, 0xff, (size_t)d * 4, st);
+    S.lv = (QLevel *)(m + lv);
+    S.stride = P.n * P.d * P.T >= PROBE_OFTEN ? 2 : 4;
+    cudaError_t e = cudaMemsetAsync(S.lv, 0, 32 * sizeof(QLevel), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(S.rng, 0xff, (size_t)d * 4, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(S.rng + d, 0, (size_t)d * 4, st);
     if (e != cudaSuccess) return e;
     const int rows = 256;
@@ -1114,29 +1172,29 @@ cudaError_t quant_level(QuantScratch &S, const BuildParams &P, int l, const int 
     const int dblocks = (S.ldq + S.tpr * 8 - 1) / (S.tpr * 8);
     const size_t smem = (size_t)2 * S.tpr * 8 * 8;
     long long *sums = S.sums[l & 1], *parent = S.sums[(l & 1) ^ 1];
-    auto qsum = [&](int mode, long long node0, long long nodes, long long slots) {
-        cudaError_t e = nch > 1 ? cudaMemsetAsync(sums, 0, (size_t)slots * P.d * 16, st) : cudaSuccess;
-        if (e != cudaSuccess) return e;
-        k_qsum<<<dim3((unsigned)(nodes * nch), dblocks), 256, smem, st>>>(P, l, mode, node0, nch, S.tpr, seq, S.xq, S.ldq, sums);
-        return cudaGetLastError();
-    };
-    auto pick = [&](long long node0, long long nodes, int derive) {
-        k_cand<<<(unsigned)nodes, NT, 0, st>>>(P, l, node0, derive, S.qdim, parent, sums, S.ncand, S.cand);
-        return cudaGetLastError();
-    };
+    if (S.first < 0) S.first = l;
+    QPlan W;
+    W.lv = S.lv;
+    W.nodes = nseg;
+    W.first = l == S.first;
+    W.keeps = nseg <= S.cap;
+    W.stride = S.stride;
     cudaError_t e = cudaSuccess;
-    if (l > 0 && S.have == l - 1 && nseg <= S.cap) {
-        // left children summed, right ones derived (both kinds write their sums before any child reads
-        // them: the left ones in the first launch)
-        if ((e = qsum(Q_LEFT, 0, nseg / 2, nseg)) == cudaSuccess) e = pick(0, nseg, 1);
-        S.have = l;
-        return e;
-    }
+    // (the left children's sums and the derived ones are all written before any child reads them: the left
+    // ones in the first launch)
     for (long long n0 = 0; n0 < nseg && e == cudaSuccess; n0 += S.cap) {
         const long long nodes = std::min(S.cap, nseg - n0);
-        if ((e = qsum(Q_FROM, n0, nodes, nodes)) == cudaSuccess) e = pick(n0, nodes, 0);
+        if (nch > 1 && (e = cudaMemsetAsync(sums, 0, (size_t)nodes * P.d * 16, st)) != cudaSuccess) break;
+        k_qsum<<<dim3((unsigned)(nodes * nch), dblocks), 256, smem, st>>>(P, W, l, n0, nch, S.tpr, seq, S.xq, S.ldq, sums);
+        k_cand<<<(unsigned)nodes, NT, 0, st>>>(P, W, l, n0, S.qdim, parent, sums, S.ncand, S.cand);
+        e = cudaGetLastError();
     }
-    if (nseg <= S.cap) S.have = l;
+    if (e == cudaSuccess && (W.first || !S.decides)) {
+        QLevel got;
+        e = cudaMemcpyAsync(&got, S.lv + l, sizeof got, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        S.decides = q_decides(got);
+    }
     return e;
 }
 
@@ -1200,7 +1258,6 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
 
     QuantScratch S;
     if (!F->U && !P.global_scope && L > 0 && n >= QMIN) GF_CUDA_TRY(quant_prepare(S, P, (long long)T << (L - 1), maxch, F->num_sms, st));
-    const int *chosen = S.on ? S.ncand : nullptr;  // >= 0: the node's split dimension is chosen below
 
     const int ndb = (F->d + DB - 1) / DB;
     for (int l = 0; l < L; ++l) {
@@ -1210,7 +1267,8 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
         if (cm <= SMALL) {
             const size_t smem = sizeof(SmallSmem) + (size_t)cm * 8;
             // (level 0 of a small set: every tree does its own root)
-            const bool sel = S.on && l > 0;
+            const bool sel = S.takes(l) && l > 0;
+            const int *chosen = sel ? S.ncand : nullptr;  // >= 0: the node's split dimension is in segs
             if (sel) {
                 GF_CUDA_TRY(quant_level(S, P, l, bufA, st));
                 k_exact<<<(unsigned)((nseg * 32 + NT - 1) / NT), NT, 0, st>>>(P, l, nseg, bufA, chosen, S.cand, S.segs);
@@ -1225,7 +1283,8 @@ static int build_levels(gf_forest *F, const gf_rand_params &rp, uint64_t seed, c
             unsigned *gh = (unsigned *)ghist.p;
             const unsigned gseg = (unsigned)((nseg + 255) / 256);
             if (!P.global_scope || l == 0) {
-                if (S.on) {
+                const int *chosen = S.takes(l) ? S.ncand : nullptr;  // >= 0: the node's split dimension is in segs
+                if (chosen) {
                     GF_CUDA_TRY(quant_level(S, P, l, bufA, st));
                     const long long own = l == 0 ? nch : nchunks;  // level 0: tree 0's chunks serve all
                     k_exact_chunk<<<(unsigned)((own * 32 + NT - 1) / NT), NT, 0, st>>>(

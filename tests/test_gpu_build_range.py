@@ -76,3 +76,32 @@ def test_builds_around_the_fixed_point_pass_smallest_size(gf, n):
     assert np.array_equal(A.split_dim, B.split_dim)
     assert np.array_equal(A.split_val, B.split_val)
     assert np.array_equal(A.perm, B.perm)
+
+
+def two_far(X):     # two far points set every dimension's step: the upper nodes stay undecided, small ones not
+    X = np.random.default_rng(1).standard_normal(X.shape).astype(np.float32)
+    X[0], X[1] = 1000.0, -1000.0
+    return X
+
+
+def one_far(X):     # no node without it tells its dimensions apart
+    X[0] = 1e6
+    return X
+
+
+def tied(X):        # three columns over and over
+    return np.tile(X[:, :3], (1, X.shape[1]))[:, :X.shape[1]]
+
+
+@pytest.mark.parametrize("change", [two_far, one_far, tied])
+@pytest.mark.parametrize("n,d,T,p", [(20_000, 300, 3, 20), (40_000, 90, 1, 9), (5000, 260, 40, 700), (3000, 600, 600, 5)])
+def test_levels_the_bounds_leave_undecided(gf, change, n, d, T, p):
+    """The pass stops where it decides too few nodes and may come back (by derived sums or direct ones; the
+    last shape has more nodes than a sums buffer)."""
+    X, _ = synth.mixture(n, d, 1, "A", seed=n)
+    X = np.ascontiguousarray(change(X))
+    _, A = gpu_build(gf, X, T, p, t=3, seed=4)
+    _, B = gpu_build(gf, X, T, p, t=3, seed=4, U=np.zeros((T, d), np.float32))
+    assert np.array_equal(A.split_dim, B.split_dim)
+    assert np.array_equal(A.split_val, B.split_val)
+    assert np.array_equal(A.perm, B.perm)
