@@ -316,7 +316,7 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 // the variance on both sides.  What has to lie between the bounds is the variance as the full sums give
 // it.  Over the up to 8192 points they add at a time, these are off by some 2^-38 of range_j^2 a point,
 // a sixtieth of s_j^2 (ROUNDED allows half of it), as long as nothing under- or overflows: for range_j
-// in [QLOW, QHIGH].  Below, squares may vanish, but the sums stay at most c (range_j^2 + 2^-147): no
+// in [QLOW, QHIGH].  Below, squares may vanish altogether, but the sums stay at most c (range_j^2 + 2^-147): no
 // lower bound, that upper one.  Above, nothing is known.  A level's sums read 2 bytes a coordinate instead of 4 and cost a few
 // integer instructions instead of some 26 of compensated float32: 500,000 x 960, T = 32, a level took
 // 15.4 ms of compensated sums (1.0e12 coordinates/s, bound by those instructions) and takes 2.1 ms of
@@ -325,7 +325,7 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 constexpr int CAND_MAX = 64;       // dimensions listed per node; -1: more, the node is summed in full
 constexpr float QERR = 0.52f;
 constexpr float QSTEPS = 65000.f;  // s_j = range_j / QSTEPS
-constexpr float QLOW = 1e-12f, QHIGH = 1e14f;  // s_j^2 2^-24 and 2^31 range_j^2 are normal floats
+constexpr float QLOW = 1e-16f, QHIGH = 1e14f;  // 2^-148, what a square may lose, is 0.2% of s_j^2; 2^31 range_j^2 is finite
 constexpr float ROUNDED = 0.5f;
 constexpr int QBIAS = 32500;       // half of them
 constexpr int QCHUNK = 2048;       // points a CTA sums
@@ -534,10 +534,10 @@ __device__ __forceinline__ void dev_bounds(long long S1, long long S2, float c, 
         return;
     }
     const float m2 = (float)S2, m1 = (float)S1;
-    const float v = m2 - m1 * (m1 / c), e = m2 * 9.5367431640625e-7f, h = QERR * sqrtf(c), s2 = s * s;
+    const float v = m2 - m1 * (m1 / c), e = m2 * 9.5367431640625e-7f, h = QERR * sqrtf(c);
     const float rl = fmaxf(sqrtf(fmaxf(v - e, 0.f)) - h, 0.f), rh = sqrtf(fmaxf(v + e, 0.f)) + h;
-    lo = fmaxf(rl * rl - ROUNDED * c, 0.f) * s2 * (1.f - 1e-5f);
-    hi = (rh * rh + ROUNDED * c) * s2 * (1.f + 1e-5f);
+    lo = fmaxf(rl * rl - ROUNDED * c, 0.f) * (1.f - 1e-5f) * s * s;  // (s * s alone may vanish)
+    hi = (rh * rh + ROUNDED * c) * (1.f + 1e-5f) * s * s;
 }
 
 // The dimensions that may be among the t of largest variance, per node: those whose upper bound

@@ -51,7 +51,7 @@ def faint(X):   # equal spreads, at which float32 keeps a few bits of the square
     return (np.random.default_rng(X.shape[0]).standard_normal(X.shape) * 1e-22).astype(np.float32)
 
 
-SCALES = [1e-12, 1e-15, 1e-18, 1e-20, 1e-22, 1e-26, 1e-37, 1e15, 1e19]
+SCALES = [1e-12, 1e-15, 1e-16, 1e-17, 1e-18, 1e-20, 1e-22, 1e-26, 1e-37, 1e15, 1e19]
 
 
 @pytest.mark.parametrize("change", SCALES + [ramp, steep, speck, faint])
