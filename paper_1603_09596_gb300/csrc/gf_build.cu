@@ -1094,13 +1094,6 @@ __global__ void k_iota(int *perm, long long n, int T) {
 struct DevBuf {
     void *p = nullptr;
     ~DevBuf() { cudaFree(p); }
-    // memory the build can do without: false (and no error left behind) if there is none
-    bool spare(size_t bytes) {
-        if (cudaMalloc(&p, bytes) == cudaSuccess) return true;
-        cudaGetLastError();
-        p = nullptr;
-        return false;
-    }
 };
 
 // Scratch of the fixed-point pass (k_qsum and after); without it the build takes the full-precision
@@ -1139,7 +1132,7 @@ cudaError_t quant_prepare(QuantScratch &S, const BuildParams &P, long long wides
     const size_t sums[2] = {place((size_t)S.cap * d * 16), place((size_t)S.cap * d * 16)};
     const size_t ncand = place((size_t)widest * 4), cand = place((size_t)widest * CAND_MAX * 4), segs = place((size_t)widest * 4);
     const size_t xpart = place((size_t)maxch * 2 * CAND_MAX * 8), lv = place(32 * sizeof(QLevel));
-    S.on = S.mem.spare(total);
+    S.on = gf_dmalloc_if(&S.mem.p, total);
     if (!S.on) return cudaSuccess;
     char *m = (char *)S.mem.p;
     S.rng = (unsigned *)(m + rng);

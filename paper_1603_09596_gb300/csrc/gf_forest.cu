@@ -42,15 +42,25 @@ extern "C" int gf_debug_fail_alloc(int32_t after) {
     return GF_OK;
 }
 
+// Whether this allocation is the one that gf_debug_fail_alloc asks to fail.
+static bool alloc_refused() {
+    for (int c = g_alloc_countdown.load(); c >= 0;)
+        if (g_alloc_countdown.compare_exchange_weak(c, c - 1)) return c == 0;
+    return false;
+}
+
+bool gf_dmalloc_if(void **p, size_t bytes) {
+    *p = nullptr;
+    if (!alloc_refused() && cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
+}
+
 int gf_dmalloc(void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return GF_OK;
-    for (int c = g_alloc_countdown.load(); c >= 0;) {
-        if (g_alloc_countdown.compare_exchange_weak(c, c - 1)) {
-            if (c == 0) return gf_fail(GF_ENOMEM, "cudaMalloc(%zu bytes): refused (gf_debug_fail_alloc)", bytes);
-            break;
-        }
-    }
+    if (alloc_refused()) return gf_fail(GF_ENOMEM, "cudaMalloc(%zu bytes): refused (gf_debug_fail_alloc)", bytes);
     cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
         *p = nullptr;

@@ -119,6 +119,8 @@ int gf_cuda_fail(cudaError_t e, const char *what);
 
 // Allocation with the library's error code (nothing is leaked on failure).
 int gf_dmalloc(void **p, size_t bytes);
+// Memory that the caller can do without: false, with no error left behind, if there is none.
+bool gf_dmalloc_if(void **p, size_t bytes);
 
 // Lets a kernel be launched with `smem` bytes of dynamic shared memory.  The limit is the kernel's, for all
 // threads of the process, so every launch sets the same one: all that the device has beside the kernel's
