@@ -2,10 +2,11 @@
 // points of the C ABI.
 #include "gf_internal.cuh"
 
-#include <atomic>
+#include "gf_squares.cuh"
 #include "gf_trace.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -391,30 +392,6 @@ extern "C" int gf_forest_set_tuning(gf_forest *F, int32_t precision, int32_t war
 
 // ---------------------------------------------------------------- screening copies
 
-// A lane's share of a row's squared norm: float32 squares (exact in range: at most 16 significant bits)
-// summed as a float32 pair and added to a float64 sum at least every 32 squares.  The float64 conversion and
-// multiply-add of every value took most of the copies' time (GB300's float64 rate).
-struct SquareSum {
-    float hi = 0.f, lo = 0.f;
-    double acc = 0.0;
-    __device__ __forceinline__ void add(float v) {
-        const float p = __fmul_rn(v, v), s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b)));
-        hi = s;
-    }
-    __device__ __forceinline__ void flush() {
-        acc += hi;
-        acc += lo;
-        hi = lo = 0.f;
-    }
-    __device__ __forceinline__ double warp_total() {
-        flush();
-        double a = acc;
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        return a;
-    }
-};
-
 // Four values of a row from column j on, zeros past d (rows are 16-byte aligned, ldx a multiple of four).
 __device__ __forceinline__ float4 row4(const float *r, int j, int d, int ldx) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -460,7 +437,7 @@ __global__ void __launch_bounds__(256) k_to_bf16(const float *__restrict__ x, in
             sum.flush();
         }
         double total = sum.warp_total();
-        if (!(total > 1e-30 && total < 1e37)) {  // squares outside float32's range: every value in float64 (uniform)
+        if (!(total > 1e-20 && total < 1e37)) {  // squares outside float32's range could count: every value in float64 (uniform)
             total = 0.0;
             for (int j = lane; j < d; j += 32) {
                 const double v = (double)__bfloat162float(__float2bfloat16_rn(__ldg(r + j)));

@@ -1,9 +1,16 @@
 """The screening copies and their norms at the ends of float32's range."""
+import ctypes as C
+import math
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
+from conftest import ROOT
 from oracle import screen
+from paper_1603_09596_gb300 import _build
 from parity import U32
 
 pytestmark = pytest.mark.gpu
@@ -36,3 +43,23 @@ def test_fp8_rows_too_small_for_the_inverse_scale(gf, d):
     for i in range(m):
         want = ((deq - Q[i].astype(np.float64)) ** 2).sum(1)
         assert np.all(np.abs(got[i] - want) <= (np.ceil(d / 32) + 16) * U32 * want)  # parity.screen_bounds, "direct"
+
+
+@pytest.mark.parametrize("d", [1, 33, 960, 3000])
+def test_sums_of_squares_round_like_float64_ones(tmp_path, d):
+    """bfloat16 values over twenty binary orders: a lane rounds three times every 32 squares (2^-53 of a sum
+    that is at most the total), and the warp five times more."""
+    lib = str(tmp_path / "squares.so")
+    subprocess.run([_build.nvcc(), "-gencode", _build.GENCODE, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-shared",
+                    "-cudart", "shared", "-I", _build.CSRC, "-o", lib,
+                    os.path.join(ROOT, "tests", "native", "square_sums.cu")], check=True)
+    rng = np.random.default_rng(d)
+    n = 300
+    X = screen.bf16_round((rng.standard_normal((n, d)) * 2.0 ** rng.uniform(-10, 10, (n, d))).astype(np.float32))
+    X = np.ascontiguousarray(X)
+    out = np.zeros(n)
+    f = C.CDLL(lib).square_sums
+    f.argtypes = [C.c_void_p, C.c_longlong, C.c_int, C.c_void_p]
+    assert f(X.ctypes.data, n, d, out.ctypes.data) == 0
+    want = np.array([math.fsum(r * r) for r in X.astype(np.float64)])
+    assert np.all(np.abs(out - want) <= (3 * -(-d // 1024) + 6) * 2.0 ** -53 * want)
