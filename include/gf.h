@@ -63,7 +63,7 @@ typedef struct gf_rand_params {
 
 /* Query kernel.  Both give the same results (same distances, same (distance, id) order). */
 #define GF_ALGO_AUTO 0   /* LEAF where the batch shares leaves enough; else, unless a workspace or a
-                            CTA shape is given, a staged path over the same candidates (scratch from
+                            CTA shape is given in the call, a staged path over the same candidates (scratch from
                             the library's pool); else SORT for small candidate bounds, STREAM otherwise */
 #define GF_ALGO_SORT 1   /* candidates sorted and de-duplicated in shared memory; needs
                             8 * next_pow2(T * max_leaf) bytes of shared memory per CTA */
@@ -227,7 +227,9 @@ int gf_forest_load(const char *path, gf_forest **out);
 int gf_forest_add_screen(gf_forest *F, int32_t precision, void *stream);
 
 /* Set the forest's default kernel shape and shortlist for one precision (what the autotuner
- * writes); gf_query_ex uses them where its options hold 0.  rerank_R / rows_in_flight 0 keep the
+ * writes); gf_query_ex uses them where its options hold 0: the shape in the kernels that have one (SORT,
+ * STREAM, and ctas_per_sm in LEAF).  GF_ALGO_AUTO chooses its path without regard to it; naming a shape in
+ * a call's options keeps that call off the staged path.  rerank_R / rows_in_flight 0 keep the
  * current value.  Limits: 1 <= warps_per_cta <= 32, 0 <= ctas_per_sm <= 32, 0 <= rerank_R <= 2048,
  * rows_in_flight 0, 2 or 4 (else GF_EINVAL); forest files are held to the same limits. */
 int gf_forest_set_tuning(gf_forest *F, int32_t precision, int32_t warps_per_cta,

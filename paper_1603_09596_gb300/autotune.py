@@ -10,7 +10,9 @@ For a resident forest and a sample of queries it
      against the exact neighbours (the library's own exact scan), are within `tol` of the float32
      search's; without X, the shortest R whose answers agree with the float32 search on at least
      `agree` of the sample's top-k entries;
-and stores the choice in the forest (gf_forest_set_tuning), where gf_query picks it up.
+and stores the choice in the forest (gf_forest_set_tuning), where the kernels that have a shape pick it
+up: the one-CTA kernels (a call with a workspace or a fixed algorithm runs them) and the leaf-major
+one.  GF_ALGO_AUTO's staged path has none; a call without a shape may take it whatever is stored.
 Results are cached per (n, d, T, leaf_size, k, precision, batch) for the process.
 """
 from __future__ import annotations
@@ -54,7 +56,8 @@ def tune(F: gf.Forest, Q: torch.Tensor, k: int, precision: int, agree: float = 0
          tol: float = 0.005, algo: int = gf.GF_ALGO_AUTO, r_max: int = 0,
          Qt: torch.Tensor | None = None) -> dict:
     """Qt: the batch the shapes are timed on (default Q); the best shape depends on how many
-    queries share a leaf, so time it on a batch of the size that will run."""
+    queries share a leaf, so time it on a batch of the size that will run.  The result's "ms" is the time of
+    gf_query without a shape on the tuned forest; with GF_ALGO_AUTO "shape_ms" is that of the shape stored."""
     inf = F.info
     Qt = Q if Qt is None else Qt
     key = (inf.n, inf.d, inf.T, inf.leaf_size, k, precision, Q.shape[0], checks, X is not None, algo, r_max,
@@ -110,6 +113,9 @@ def tune(F: gf.Forest, Q: torch.Tensor, k: int, precision: int, agree: float = 0
     res.update(warps=w, ctas_per_sm=c, rows_in_flight=g, ms=t,
                timings={f"{a}x{b}x{e}": v for (a, b, e), v in timings.items()})
     gf.gf_forest_set_tuning(F, precision, w, c, R, g)
+    if algo == gf.GF_ALGO_AUTO:  # what a call that names no shape takes from now on
+        res["shape_ms"] = t
+        res["ms"] = _time(lambda: gf.gf_query(F, Qt, k, precision=precision, rerank_R=R, checks=checks))
     _cache[key] = res
     return res
 

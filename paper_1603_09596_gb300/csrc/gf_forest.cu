@@ -565,7 +565,7 @@ extern "C" int gf_query_ex(const gf_forest *F, const float *Q, int64_t m, int32_
     if (o->checks < 0 || !(o->eps >= 0.0)) return gf_fail(GF_EINVAL, "checks < 0 or eps < 0");
     x.leaf_budget = leaf_budget_of(F, o->checks, o->eps);
     x.events = (cudaEvent_t *)o->events;
-    x.shaped = o->warps_per_cta > 0 || o->ctas_per_sm > 0 || o->rows_in_flight > 0 || warps > 8;
+    x.shaped = o->warps_per_cta > 0 || o->ctas_per_sm > 0 || o->rows_in_flight > 0;
     if (x.leaf_budget > 0) {
         if (((unsigned long long)F->T << F->L) > 0xffffffffull)
             return gf_fail(GF_EUNSUPPORTED, "priority search needs T * 2^L <= 2^32");

@@ -150,7 +150,7 @@ struct QueryExtra {
     int32_t order = GF_ORDER_AUTO;
     int32_t leaf_budget = 0;  // leaves per query for the priority search (0: one per tree)
     cudaEvent_t *events = nullptr;  // recorded around the scoring kernel's launches (timing)
-    bool shaped = false;            // the caller (or the forest's tuning) asks for a CTA shape of the one-CTA kernels
+    bool shaped = false;            // the call (not the forest's tuning) names a CTA shape of the one-CTA kernels
 };
 
 // Record events[i] on st when the caller asked for timing events.

@@ -90,3 +90,24 @@ def test_routes_of_few_candidates_answer_alike(gf, prec, n, d, T, p, m, k):
         for algo in (gf.GF_ALGO_SORT, gf.GF_ALGO_STREAM):
             b = gf.gf_query(F, Qg, k, precision=P, rerank_R=R, algo=algo)
             assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+def test_tuning_leaves_autos_path_alone(gf):
+    """A small batch on a forest tuned to any shape takes the path, and the time, of an untuned one: the
+    staged steps are some five times as fast here as the one-CTA kernels with any shape."""
+    from paper_1603_09596_gb300 import autotune
+    X, Q = synth.mixture(50_000, 512, 27, "B", seed=85, qseed=86)
+    Xg, Qg = torch.from_numpy(X).cuda(), torch.from_numpy(Q).cuda()
+
+    def ms(F, **kw):
+        return autotune._time(lambda: gf.gf_query(F, Qg, 10, **kw), reps=9)
+
+    F = gf.gf_build(Xg, 16, 256, seed=1)
+    plain, sort = ms(F), ms(F, algo=gf.GF_ALGO_SORT)
+    assert sort > 2.5 * plain
+    for shape in ((16, 0, 0, 0), (4, 2, 0, 2), (8, 1, 0, 0)):
+        gf.gf_forest_set_tuning(F, gf.GF_FP32, *shape)
+        assert ms(F) < 1.5 * plain
+    res = autotune.tune(F, Qg, 10, gf.GF_FP32)
+    assert res["ms"] < 1.5 * plain < res["shape_ms"]
+    assert ms(F) < 1.5 * plain
