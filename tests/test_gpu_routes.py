@@ -111,3 +111,21 @@ def test_tuning_leaves_autos_path_alone(gf):
     res = autotune.tune(F, Qg, 10, gf.GF_FP32)
     assert res["ms"] < 1.5 * plain < res["shape_ms"]
     assert ms(F) < 1.5 * plain
+
+
+# Device bitmaps in three waves of reordered queries (n above 1.8 million, T ceil(n / 2^L) above 8192), and the
+# single launch with rows of 513 to 1024 dimensions.
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8"])
+@pytest.mark.parametrize("n,d,T,p,m,k", [(2_000_000, 4, 20, 1000, 1500, 33), (3000, 600, 8, 50, 200, 10), (3000, 1024, 8, 50, 200, 10)])
+def test_staged_path_in_its_less_usual_forms(gf, prec, n, d, T, p, m, k):
+    X, Q = synth.mixture(n, d, m, "A", seed=87, qseed=88)
+    F = gf.gf_build(torch.from_numpy(X).cuda(), T, p, t=min(5, d), seed=1)
+    P, R = gf.PRECISIONS[prec], 0 if prec == "fp32" else 40
+    if P:
+        gf.gf_forest_add_screen(F, P)
+    Qg = torch.from_numpy(Q).cuda()
+    counts = [torch.zeros(m, dtype=torch.int32, device="cuda") for _ in range(2)]
+    # (asking for the candidates' number keeps a batch off the leaf-major path)
+    a = gf.gf_query(F, Qg, k, precision=P, rerank_R=R, ncand_out=counts[0])
+    b = gf.gf_query(F, Qg, k, precision=P, rerank_R=R, algo=gf.GF_ALGO_STREAM, ncand_out=counts[1])
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and torch.equal(counts[0], counts[1])
