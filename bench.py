@@ -12,7 +12,7 @@ the float32-only path and the tree parameters T=32, leaf_size=64 are reported be
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--small]
 
-Prints one JSON line (rank 0).
+Prints one JSON line on standard output (rank 0); the figures behind it go to standard error.
 """
 from __future__ import annotations
 
@@ -646,9 +646,29 @@ def ours(args):
         "p99_ms": lat["p99_ms"] if lat else None,
     }
     if rank == 0:
-        print(json.dumps(line))
+        short, detail = contract_line(line)
+        print(json.dumps({"detail": detail}), file=sys.stderr, flush=True)
+        print(json.dumps(short))
     if world > 1:
         torch.distributed.destroy_process_group()
+
+
+# What standard output's one line holds; everything else goes to standard error.  (A reader that keeps
+# the last few KB of the output has to find the whole line in them.)
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "gpu_launches", "config", "roofline", "cpu_baseline", "clocks", "e2e",
+             "p99_ms")
+ROOFLINE_KEYS = ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_kind", "kernel", "kernel_ms", "step_ms")
+
+
+def contract_line(line):
+    """(the line's keys, the rest): of the roofline and the CPU baseline the line holds the figures only."""
+    short = {key: line[key] for key in LINE_KEYS if key in line}
+    if short.get("roofline"):
+        short["roofline"] = {key: v for key, v in short["roofline"].items() if key in ROOFLINE_KEYS}
+    if short.get("cpu_baseline"):
+        short["cpu_baseline"] = {key: v for key, v in short["cpu_baseline"].items() if not isinstance(v, dict)}
+    return short, {key: v for key, v in line.items() if key not in short or short[key] != v}
 
 
 def cpu_baseline(X, Q, F, gf, k, budget_s=15.0, checks=0):
