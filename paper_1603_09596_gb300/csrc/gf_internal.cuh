@@ -196,8 +196,6 @@ const char *gf_leaf_unsupported(const gf_forest *F, int64_t m, int32_t k, int32_
 bool gf_list_usable(const gf_forest *F, int64_t m, int32_t k, int32_t precision, int32_t R, const QueryExtra &x);
 int gf_launch_list(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision, int32_t R, bool sorts,
                    cudaStream_t st, int64_t *ids, float *dists, const QueryExtra &x, bool *ran);
-// order[0..m) = the queries of okeys (leaf << 32 | query) sorted, in chunks of 16,384
-cudaError_t gf_sort_order(int64_t m, const unsigned long long *okeys, int *order, cudaStream_t st);
 
 // Per-call device scratch, stream-ordered, from a pool of the library's own that keeps up to 1 GiB
 // between calls (the default pool gives everything back at each synchronization, and mapping it

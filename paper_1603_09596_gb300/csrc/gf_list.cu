@@ -709,7 +709,7 @@ cudaError_t one_prec(const gf_forest *F, const float *Q, int64_t m, int k, int k
     if constexpr (PREC == P_F32) {
         GF_ONE(1, 1) GF_ONE(2, 2) GF_ONE(4, 4) GF_ONE(8, 8)
     } else {
-        GF_ONE(1, 1) GF_ONE(1, 2) GF_ONE(1, 4) GF_ONE(2, 4) GF_ONE(2, 8) GF_ONE(4, 8) GF_ONE(1, 8)
+        GF_ONE(1, 1) GF_ONE(1, 2) GF_ONE(1, 4) GF_ONE(2, 4) GF_ONE(2, 8) GF_ONE(4, 8)
     }
 #undef GF_ONE
     return cudaErrorInvalidValue;

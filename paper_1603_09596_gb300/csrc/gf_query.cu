@@ -699,6 +699,16 @@ StreamWorkspace stream_workspace(const gf_forest *F, long long m, long long grid
     return W;
 }
 
+// order[0..m) = the queries of okeys (leaf << 32 | query) sorted, in chunks of 16,384
+cudaError_t sort_order(int64_t m, const unsigned long long *okeys, int *order, cudaStream_t st) {
+    const long long chunks = (m + ORDER_CHUNK - 1) / ORDER_CHUNK;
+    const size_t smem = (size_t)next_pow2((int)std::min<long long>(m, ORDER_CHUNK)) * 8;
+    const cudaError_t e = gf_smem_limit((const void *)k_order_sort, smem);
+    if (e != cudaSuccess) return e;
+    k_order_sort<<<(unsigned)chunks, 1024, smem, st>>>(m, okeys, order);
+    return cudaGetLastError();
+}
+
 // buffer: the kept keys plus one phase of appends
 int stream_buf_len(int keep) { return keep + LIST; }
 
@@ -772,7 +782,7 @@ int launch_stream_g(const gf_forest *F, const float *Q, int64_t m, int32_t k, in
         unsigned long long *okeys = (unsigned long long *)((char *)bitmaps + W.okeys);
         order = (int *)((char *)bitmaps + W.order);
         k_order_keys<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(view_of(F), Q, m, okeys);
-        const cudaError_t eo = gf_sort_order(m, okeys, order, st);
+        const cudaError_t eo = sort_order(m, okeys, order, st);
         if (eo != cudaSuccess) {
             if (own) gf_scratch_free(bitmaps, st);
             return gf_cuda_fail(eo, "query order");
@@ -854,15 +864,6 @@ int dispatch_prec(const gf_forest *F, const float *Q, int64_t m, int32_t k, int3
 }
 
 }  // namespace
-
-cudaError_t gf_sort_order(int64_t m, const unsigned long long *okeys, int *order, cudaStream_t st) {
-    const long long chunks = (m + ORDER_CHUNK - 1) / ORDER_CHUNK;
-    const size_t smem = (size_t)next_pow2((int)std::min<long long>(m, ORDER_CHUNK)) * 8;
-    const cudaError_t e = gf_smem_limit((const void *)k_order_sort, smem);
-    if (e != cudaSuccess) return e;
-    k_order_sort<<<(unsigned)chunks, 1024, smem, st>>>(m, okeys, order);
-    return cudaGetLastError();
-}
 
 int gf_launch_query(const gf_forest *F, const float *Q, int64_t m, int32_t k, int32_t precision,
                     int32_t R, int32_t warps, int32_t ctas_per_sm, cudaStream_t st, int64_t *ids,
