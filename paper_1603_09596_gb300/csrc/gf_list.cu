@@ -23,8 +23,10 @@
 //   2000 queries, 2 10^5 x 10^4, T = 24, p = 32, E4M3               3173 -> 2238 (sort)
 //   10^4 queries, 10^6 x 960, T = 32, p = 64, bf16 (1.24k rows)     8798 -> 3037 (sort)
 //   5003 queries, 7 10^5 x 101, T = 32, p = 64, float32              890 -> 419  (sort)
-// The scoring step is bound by the row loads: 9.8 TB/s of rows at 10^4 queries (most from L2, whose
-// register loads peak at 10.6 TB/s), 7.2 TB/s at 199 queries (HBM).
+// The scoring step is bound by the row loads: 9.8 TB/s of rows at 10^4 queries, of which HBM serves 3.9
+// (ncu) and L2 the rest, whose register loads peak at 10.6 TB/s; 7.2 TB/s at 199 queries, 6.5 of them from
+// HBM (the 0.96 GB of the copy are read almost twice: half of the repeats miss L2); E4M3 rows of 10^4
+// bytes 4.8 TB/s from HBM, which is not at its limit there.
 #include "gf_internal.cuh"
 #include "gf_device.cuh"
 #include "gf_score.cuh"
@@ -762,7 +764,10 @@ namespace {
 // Whether work on st goes into a graph.
 bool captured(cudaStream_t st) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) cudaGetLastError();
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {  // the legacy stream beside another's capture: the launches report it
+        cudaGetLastError();
+        return false;
+    }
     return status != cudaStreamCaptureStatusNone;
 }
 
