@@ -95,10 +95,12 @@ typedef struct gf_query_opts {
     void *stream;            /* cudaStream_t */
     int32_t algo;            /* GF_ALGO_* */
     int32_t rows_in_flight;  /* STREAM only: rows each warp scores at once, 2 or 4; 0 = default */
-    void *workspace;         /* STREAM only: device scratch of at least gf_query_workspace_size()
+    void *workspace;         /* STREAM, LEAF: device scratch of at least gf_query_workspace_size()
                                 bytes, zero-filled before its first use (every query leaves it zero
-                                again); NULL = the library allocates it stream-ordered
-                                (cudaMallocAsync / cudaFreeAsync) for this call */
+                                again); NULL = the library allocates it stream-ordered for this call
+                                from a memory pool of its own, which keeps up to 1 GiB between calls
+                                while a forest lives (not part of device_bytes).  With a workspace
+                                AUTO takes the one-CTA kernels or LEAF, never the staged path */
     int64_t workspace_bytes; /* size of `workspace` */
     int32_t *ncand_out;      /* STREAM only, optional: device [m] int32, number of distinct
                                 candidates of each query */
@@ -110,7 +112,10 @@ typedef struct gf_query_opts {
                                 query records events[0] on `stream` just before the first launch of
                                 its scoring kernel (k_leaf_score / k_leaf_f32 on the leaf-major path,
                                 else the streaming or sort query kernel) and events[1] just after the
-                                last, so that kernel can be timed alone; NULL: no events */
+                                last, so that kernel can be timed alone; on the staged path they span
+                                the admission and the scoring of all its waves (and, for calls below
+                                512 queries, the descents; with several waves the selections of all but
+                                the last; in the single launch the whole search); NULL: no events */
 } gf_query_opts;
 
 typedef struct gf_forest gf_forest; /* opaque; owned by the library */
@@ -124,7 +129,7 @@ typedef struct gf_forest_info {
     int32_t max_leaf;    /* ceil(n / 2^L) */
     int32_t cand_cap;    /* T * max_leaf: upper bound on candidates per query */
     int32_t screens;     /* bit (1 << GF_BF16_RERANK) / (1 << GF_FP8_RERANK): derived copies held */
-    int64_t device_bytes;/* device memory owned by the forest */
+    int64_t device_bytes;/* device memory owned by the forest (the queries' scratch is not) */
 } gf_forest_info;
 
 void gf_rand_params_default(gf_rand_params *rp); /* t = 5, shuffle = 1, var_scope = NODE */

@@ -320,8 +320,8 @@ __device__ void block_partition(const int *__restrict__ rows, const unsigned lon
 // lower bound, that upper one.  Above, nothing is known.  A level's sums read 2 bytes a coordinate instead of 4 and cost a few
 // integer instructions instead of some 26 of compensated float32: 500,000 x 960, T = 32, a level took
 // 15.4 ms of compensated sums (1.0e12 coordinates/s, bound by those instructions) and takes 2.1 ms of
-// k_qsum over half the points (7.4 TB/s of rows: HBM) and 0.8 ms of k_exact; the build with its bf16
-// copy and the export 174.8 -> 49.6 ms (46.6 with the copies made in one pass each).
+// k_qsum over half the points (7.4 TB/s of rows, 6.8 of them from HBM: its limit) and 0.7 to 1.1 ms of the
+// listed dimensions; the build with its bf16 copy and the export 174.6 -> 44.8 ms.
 constexpr int CAND_MAX = 64;       // dimensions listed per node; -1: more, the node is summed in full
 constexpr float QERR = 0.52f;
 constexpr float QSTEPS = 65000.f;  // s_j = range_j / QSTEPS
