@@ -63,8 +63,10 @@ typedef struct gf_rand_params {
 
 /* Query kernel.  Both give the same results (same distances, same (distance, id) order). */
 #define GF_ALGO_AUTO 0   /* LEAF where the batch shares leaves enough; else, unless a workspace or a
-                            CTA shape is given in the call, a staged path over the same candidates (scratch from
-                            the library's pool); else SORT for small candidate bounds, STREAM otherwise */
+                            CTA shape is given in the call, a staged path over the same candidates (scratch
+                            from the library's pool; not for searches of a few dozen candidates, nor under
+                            stream capture where SORT can answer); else SORT for small candidate bounds,
+                            STREAM otherwise */
 #define GF_ALGO_SORT 1   /* candidates sorted and de-duplicated in shared memory; needs
                             8 * next_pow2(T * max_leaf) bytes of shared memory per CTA */
 #define GF_ALGO_STREAM 2 /* candidates de-duplicated through a per-CTA bitmap over the point ids
